@@ -462,7 +462,13 @@ rsi_status rsi_bvh_export(rsi_bvh h, rsi_stream s, float* bounds, uint32_t* code
         rsi_status st = boxes(tb.lbox, N, lbox);
         if (st != RSI_OK) return st;
     }
-    if (nodes) RSI_CK(cudaMemcpy(nodes, tb.nodes, 64 * N, cudaMemcpyDeviceToHost));
+    if (nodes) {
+        RSI_CK(cudaMemcpy(nodes, tb.nodes, 64 * N, cudaMemcpyDeviceToHost));
+        int32_t* p = (int32_t*)nodes;
+        for (int64_t i = 0; i < N; ++i)  // leaf references are kept inverted on the device
+            for (int k = 12; k < 14; ++k)
+                if (p[16 * i + k + 2] > 0) p[16 * i + k] = ~p[16 * i + k];
+    }
     return RSI_OK;
 }
 
@@ -500,6 +506,8 @@ static rsi_status intersect_impl(rsi_bvh h, const float* dA, const float* dB, in
     else
         P.root = (int)(h->nT - 1);
     P.root4 = h->nT > 0 ? (int)(h->nT - 1) : rsi::kNoRoot;
+    P.leaf_size = h->leaf;
+    P.nT = (int)h->nT;
     P.nodes = h->tb.nodes;
     P.nodes4 = h->tb.nodes4;
     P.tris = h->tb.tris;
@@ -916,11 +924,24 @@ struct rsi_batch_s {
     rsi::BatchTile* d_tiles = nullptr;
     LaunchCfg cfg;
     int32_t leaf = 1;
+    bool walk = false;  // the phased loop takes every item
+    int64_t mode_first[3] = {0, 0, 0}, mode_tiles[3] = {0, 0, 0};
+    rsi::BatchFork fork{};
     cudaStream_t cap = nullptr;
     cudaGraphExec_t g_full = nullptr, g_trav = nullptr;
     cudaStream_t stream = nullptr;
     rsi::AllocHooks hooks{};  // device allocator of all this batch's memory
 };
+
+// The batch's own streams and events (those that were made).
+static void batch_streams_free(rsi_batch b) {
+    if (b->cap) cudaStreamDestroy(b->cap);
+    if (b->fork.start) cudaEventDestroy(b->fork.start);
+    for (int q = 0; q < 2; ++q) {
+        if (b->fork.aux[q]) cudaStreamDestroy(b->fork.aux[q]);
+        if (b->fork.done[q]) cudaEventDestroy(b->fork.done[q]);
+    }
+}
 
 extern "C" {
 
@@ -970,9 +991,15 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         const double w = items[k].mode == RSI_MODE_BOOL ? 1.0 : 1.5;
         return w * std::log2(2.0 + (double)items[k].nT);
     };
-    std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return cost(x) > cost(y); });
+    // grouped by mode (the phased loop runs one launch per mode)
+    std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) {
+        if (items[x].mode != items[y].mode) return items[x].mode > items[y].mode;
+        return cost(x) > cost(y);
+    });
     std::vector<rsi::BatchItemDev> dev(n);
     std::vector<rsi::BatchTile> tiles;
+    bool walk = true;
+    int64_t mode_first[3] = {0, 0, 0}, mode_tiles[3] = {0, 0, 0};
     for (int q = 0; q < n; ++q) {
         const int k = ord[q];
         const rsi_batch_item& it = items[k];
@@ -981,9 +1008,12 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         d.B = it.dB;
         d.nR = it.nR;
         d.root = it.nT > 0 ? (int)(table[k].off + it.nT - 1) : rsi::kNoRoot;
+        d.start = rsi::walk_start(table[k].off, (int)it.nT, leaf);
+        walk = walk && rsi::walk_fits(it.nR, N, leaf);
         d.mode = it.mode;
         d.out = trav_out((rsi_mode)it.mode, &it.out);
         for (int64_t lo = 0; lo < it.nR; lo += rsi::kBatchTile) {
+            if (mode_tiles[it.mode]++ == 0) mode_first[it.mode] = (int64_t)tiles.size();
             rsi::BatchTile t;
             t.item = k;
             t.pad = 0;
@@ -1000,6 +1030,11 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
     b->items.assign(items, items + n);
     b->cfg = cfg;
     b->leaf = leaf;
+    b->walk = walk;
+    for (int m = 0; m < 3; ++m) {
+        b->mode_first[m] = mode_first[m];
+        b->mode_tiles[m] = mode_tiles[m];
+    }
     b->n_tiles = (int64_t)tiles.size();
     TreeBufs tb;
     memset(&tb, 0, sizeof(tb));
@@ -1041,8 +1076,15 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
     if (e == cudaSuccess) e = cudaMemsetAsync(tb.status, 0, 4, cs);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cs);  // host tables go out of scope
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork.start, cudaEventDisableTiming);
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+        e = cudaStreamCreateWithFlags(&b->fork.aux[q], cudaStreamNonBlocking);
+        if (e == cudaSuccess)
+            e = cudaEventCreateWithFlags(&b->fork.done[q], cudaEventDisableTiming);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
+        batch_streams_free(b);
         rsi::dev_free(b->hooks, b->mem, cs);
         delete b;
         return RSI_ERR_CUDA;
@@ -1088,7 +1130,13 @@ rsi_status rsi_batch_intersect(rsi_batch b, rsi_stream s) {
     P.work = b->work;
     P.max_visits = b->tb.N + 2;
     P.status = b->tb.status;
-    RSI_CK(rsi::launch_batch(P, b->cfg.block, b->cfg.stack, (cudaStream_t)s));
+    P.leaf_size = b->leaf;
+    P.walk = b->walk;
+    for (int m = 0; m < 3; ++m) {
+        P.mode_first[m] = b->mode_first[m];
+        P.mode_tiles[m] = b->mode_tiles[m];
+    }
+    RSI_CK(rsi::launch_batch(P, b->cfg.block, b->cfg.stack, (cudaStream_t)s, b->fork));
     return RSI_OK;
 }
 
@@ -1131,7 +1179,7 @@ rsi_status rsi_batch_destroy(rsi_batch b) {
     if (b->g_trav) cudaGraphExecDestroy(b->g_trav);
     cudaStreamSynchronize(b->stream);
     cudaError_t e = rsi::dev_free(b->hooks, b->mem, b->stream);
-    if (b->cap) cudaStreamDestroy(b->cap);
+    batch_streams_free(b);
     delete b;
     if (e != cudaSuccess) {
         cudaGetLastError();

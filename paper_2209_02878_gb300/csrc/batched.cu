@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "rsi_trace.h"
+#include "walk.cuh"
 
 namespace rsi {
 
@@ -65,6 +66,52 @@ __global__ void __maxnreg__(128) k_batch(BatchParams P) {
     }
 }
 
+// The phased loop (walk.cuh), for the default stack: one kernel per mode over
+// that mode's tiles, so that each keeps its own register count.  Inlined into
+// one kernel the three need 128 registers: 1,790 us on 16 meshes with 3.5M
+// segments, and 2,178 us out of line (the calls save too much); the general
+// loop, inlined at 128, 2,265 us.
+template <int MODE, bool LEAFN>
+__global__ void __maxnreg__(kWalkRegs) k_batch_walk(BatchParams P) {
+    extern __shared__ float4 stage4[];
+    WalkStage& sg = ((WalkStage*)stage4)[threadIdx.x >> 5];
+    TravStats st = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+    unsigned long long segs = 0;
+    const int lane = threadIdx.x & 31;
+    TraceCtx C;
+    C.nodes = P.nodes;
+    C.tris = P.tris;
+    C.max_visits = P.max_visits;
+    C.fetch = kFetchChunk;  // unused: each tile is one warp's whole pool
+    C.ready = nullptr;
+    C.ready_chunk = 1;
+    C.wait_polls = kWaitPolls;
+    C.order = nullptr;
+    C.status = P.status;
+    while (true) {
+        unsigned long long t = 0ull;
+        if (lane == 0) t = atomicAdd(P.work + MODE, 1ull);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= (unsigned long long)P.mode_tiles[MODE]) break;
+        const BatchTile tile = P.tiles[P.mode_first[MODE] + t];
+        const BatchItemDev& it = P.items[tile.item];
+        C.A = it.A;
+        C.B = it.B;
+        C.nR = it.nR;
+        C.out = it.out;
+        walk_loop<MODE, false, LEAFN>(C, sg, it.start, nullptr, tile.lo, tile.hi, st, segs);
+    }
+}
+
+using BatchFn = void (*)(BatchParams);
+static BatchFn batch_walk_kernel(int mode, bool leafn) {
+    if (mode == RSI_MODE_BOOL)
+        return leafn ? k_batch_walk<RSI_MODE_BOOL, true> : k_batch_walk<RSI_MODE_BOOL, false>;
+    if (mode == RSI_MODE_COUNT)
+        return leafn ? k_batch_walk<RSI_MODE_COUNT, true> : k_batch_walk<RSI_MODE_COUNT, false>;
+    return leafn ? k_batch_walk<RSI_MODE_NEAREST, true> : k_batch_walk<RSI_MODE_NEAREST, false>;
+}
+
 // Zero the compaction counters of the items that compact.
 __global__ void k_zero_counts(const BatchItemDev* items, int n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -79,18 +126,60 @@ const void* batch_kernel(int stack) {
     }
 }
 
-cudaError_t launch_batch(const BatchParams& P, int block, int stack, cudaStream_t s) {
+static int batch_grid(int64_t n_tiles, int block, int grid) {
+    const int64_t need = (n_tiles + block / 32 - 1) / (block / 32);
+    return need < grid ? (int)need : grid;
+}
+
+// The modes run side by side (fork / join on aux streams): each grid fills the
+// device, so the blocks of the next mode start as those of the one before
+// run out of tiles.
+static cudaError_t launch_batch_walk(const BatchParams& P, int block, cudaStream_t s,
+                                     const BatchFork& fk) {
+    int used = 0;  // modes launched so far; the first stays on s
+    for (int mode = 2; mode >= 0; --mode) {  // NEAREST, the dearest, first
+        if (P.mode_tiles[mode] == 0) continue;
+        BatchFn fn = batch_walk_kernel(mode, P.leaf_size > 1);
+        const int bl = max_block((const void*)fn, block);
+        const int smem = (bl / 32) * (int)sizeof(WalkStage);
+        int grid = 0;
+        cudaError_t e = occupancy_grid((const void*)fn, bl, smem, &grid);
+        if (e != cudaSuccess) return e;
+        cudaStream_t q = s;
+        if (used > 0) {
+            q = fk.aux[used - 1];
+            e = cudaStreamWaitEvent(q, fk.start, 0);
+            if (e != cudaSuccess) return e;
+        } else {
+            e = cudaEventRecord(fk.start, s);
+            if (e != cudaSuccess) return e;
+        }
+        fn<<<batch_grid(P.mode_tiles[mode], bl, grid), bl, smem, q>>>(P);
+        e = cudaGetLastError();
+        if (used > 0) {  // join even when the launch failed: s must not run ahead
+            cudaError_t j = cudaEventRecord(fk.done[used - 1], q);
+            if (j == cudaSuccess) j = cudaStreamWaitEvent(s, fk.done[used - 1], 0);
+            if (e == cudaSuccess) e = j;
+        }
+        if (e != cudaSuccess) return e;
+        ++used;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_batch(const BatchParams& P, int block, int stack, cudaStream_t s,
+                         const BatchFork& fk) {
     if (P.n_tiles == 0) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(P.work, 0, 3 * sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
+    k_zero_counts<<<(P.n_items + 255) / 256, 256, 0, s>>>(P.items, P.n_items);
+    if (P.walk && stack == 64) return launch_batch_walk(P, block, s, fk);
     const void* fn = batch_kernel(stack);
     block = max_block(fn, block);
     int grid = 0;
-    cudaError_t e = occupancy_grid(fn, block, 0, &grid);
+    e = occupancy_grid(fn, block, 0, &grid);
     if (e != cudaSuccess) return e;
-    const int64_t blocks_needed = (P.n_tiles + block / 32 - 1) / (block / 32);
-    if (blocks_needed < grid) grid = (int)blocks_needed;
-    e = cudaMemsetAsync(P.work, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    k_zero_counts<<<(P.n_items + 255) / 256, 256, 0, s>>>(P.items, P.n_items);
+    grid = batch_grid(P.n_tiles, block, grid);
     switch (stack) {
         case 8: k_batch<8><<<grid, block, 0, s>>>(P); break;
         case 32: k_batch<32><<<grid, block, 0, s>>>(P); break;

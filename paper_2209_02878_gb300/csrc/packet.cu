@@ -104,7 +104,8 @@ __global__ void __maxnreg__(PacketRegs<MODE>::value) k_trace_packet(TraceParams 
                 if (STATS) ++st.visits;
                 slab2(s, q0, q1, q2, tlim, h0, t0, h1, t1);
             }
-            const int r0 = rc.x, r1 = rc.y, c0 = rc.z, c1 = rc.w;
+            const int c0 = rc.z, c1 = rc.w;
+            const int r0 = c0 > 0 ? ~rc.x : rc.x, r1 = c1 > 0 ? ~rc.y : rc.y;
             if (MODE == RSI_MODE_NEAREST) {
                 if (h0 && c0 > 0)
                     leaf_test<MODE, STATS>(s, C.A, C.B, i, C.tris, r0, c0, 0, 0, res, tlim, st);

@@ -21,7 +21,7 @@
 //                      {c0.hi.y, c1.hi.y, c0.hi.z, c1.hi.z}
 //                      {ref0, ref1, cnt0, cnt1} as int bit patterns
 //                    cnt > 0: leaf of cnt triangles starting at sorted
-//                    position ref; cnt == 0: internal slot ref; cnt == -1:
+//                    position ~ref; cnt == 0: internal slot ref; cnt == -1:
 //                    treelet node ref (only inside the treelet copy).
 //                    Slot off+n-1 is the root slot (the paper keeps its root
 //                    pointer in internalNodes[N_t-1] the same way, Sec. 3.1):
@@ -310,7 +310,8 @@ __device__ __forceinline__ void slab2(const Seg& s, const ulonglong2& q0, const 
 // errors against the exact values, (B_x + |x~| B_det) / (|det~| - B_det)
 // plus the two roundings of x~ = n_x * fl(1 / |det~|), from the bounds of
 // the stage that decided.
-__device__ __forceinline__ int mt32(const Seg& s, const float4& A, const float4& B,
+template <typename S>
+__device__ __forceinline__ int mt32(const S& s, const float4& A, const float4& B,
                                     const float4& C, bool want, float& t, float& u, float& v,
                                     float& err) {
     const float e1x = B.x - A.x, e1y = B.y - A.y, e1z = B.z - A.z;
@@ -439,7 +440,8 @@ static __device__ __noinline__ int mt64(float ax_, float ay_, float az_, float b
 // use.  Returns the bound on |t~ - t| and, in euv, the bound on
 // max(|u~ - u|, |v~ - v|), with the FP32 values; +inf when det cannot be
 // bounded away from zero.
-__device__ __forceinline__ float mt32_tight(const Seg& s, const float4& A, const float4& B,
+template <typename S>
+__device__ __forceinline__ float mt32_tight(const S& s, const float4& A, const float4& B,
                                            const float4& C, float& t, float& u, float& v,
                                            float& euv) {
     const float e1x = B.x - A.x, e1y = B.y - A.y, e1z = B.z - A.z;

@@ -25,6 +25,8 @@ struct TraceParams {
     int64_t nR;
     int root;   // treelet node ~0, a global root slot, or kNoRoot
     int root4;  // root slot for 4-wide traversal
+    int leaf_size;  // of the built tree
+    int nT;         // triangles
     const float4* nodes;
     const float4* nodes4;
     const float4* tris;
@@ -86,7 +88,8 @@ struct BatchItemDev {
     const float* A;
     const float* B;
     int64_t nR;
-    int root;  // root slot of the item's mesh, or kNoRoot
+    int root;   // root slot of the item's mesh, or kNoRoot
+    int start;  // first item of the phased loop (walk_start)
     int mode;
     TravOut out;
 };
@@ -110,9 +113,25 @@ struct BatchParams {
     unsigned long long* work;
     int max_visits;
     int32_t* status;
+    int leaf_size;  // of the built trees
+    bool walk;      // every item fits the phased loop (walk_fits)
+    // tiles of each mode: contiguous in `tiles`, one work counter each
+    int64_t mode_first[3], mode_tiles[3];
 };
 
-cudaError_t launch_batch(const BatchParams& P, int block, int stack, cudaStream_t s);
+// Streams and events for the modes' launches side by side.
+struct BatchFork {
+    cudaStream_t aux[2];
+    cudaEvent_t start, done[2];
+};
+
+// Whether the phased loop (walk.cuh) can take nR segments against trees of n
+// triangles in all, and its first item for a mesh of n triangles at off.
+bool walk_fits(int64_t nR, int64_t n, int leaf_size);
+int walk_start(int off, int n, int leaf_size);
+
+cudaError_t launch_batch(const BatchParams& P, int block, int stack, cudaStream_t s,
+                         const BatchFork& fk);
 const void* batch_kernel(int stack);
 
 }  // namespace rsi

@@ -8,7 +8,7 @@
 #include <mutex>
 
 #include "rsi_trace.h"
-#include "traverse_core.cuh"
+#include "walk.cuh"
 
 namespace rsi {
 
@@ -55,6 +55,7 @@ __global__ void __maxnreg__(TraceRegs<MODE>::value) k_trace(TraceParams P) {
     if (STATS) flush_stats(st, P.stats, segs);
 }
 
+// The default path (see walk.cuh).
 using KernelFn = void (*)(TraceParams);
 
 template <int MODE, bool STATS, int W, bool TL>
@@ -85,6 +86,58 @@ KernelFn trace_kernel(int mode, int stack, bool stats, int width, bool treelet) 
     if (treelet)
         return stats ? pick_mode<true, 2, true>(mode, stack) : pick_mode<false, 2, true>(mode, stack);
     return stats ? pick_mode<true, 2, false>(mode, stack) : pick_mode<false, 2, false>(mode, stack);
+}
+
+template <int MODE, bool STATS, bool LEAFN>
+__global__ void __maxnreg__(kWalkRegs) k_walk(TraceParams P) {
+    extern __shared__ float4 stage4[];
+    TraceCtx C;
+    C.A = P.A;
+    C.B = P.B;
+    C.nR = P.nR;
+    C.nodes = P.nodes;
+    C.tris = P.tris;
+    C.max_visits = P.max_visits;
+    C.fetch = P.fetch;
+    C.ready = P.ready;
+    C.ready_chunk = P.ready_chunk;
+    C.wait_polls = P.wait_polls > 0 ? P.wait_polls : kWaitPolls;
+    C.order = P.order;
+    C.status = P.status;
+    C.out = P.out;
+    TravStats st = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+    unsigned long long segs = 0;
+    WalkStage& sg = ((WalkStage*)stage4)[threadIdx.x >> 5];
+    walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, P.work, 0, P.nR, st, segs);
+    if (STATS) flush_stats(st, P.stats, segs);
+}
+
+template <bool STATS, bool LEAFN>
+static KernelFn pick_walk(int mode) {
+    if (mode == RSI_MODE_BOOL) return k_walk<RSI_MODE_BOOL, STATS, LEAFN>;
+    if (mode == RSI_MODE_COUNT) return k_walk<RSI_MODE_COUNT, STATS, LEAFN>;
+    return k_walk<RSI_MODE_NEAREST, STATS, LEAFN>;
+}
+
+static KernelFn walk_kernel(int mode, bool stats, bool leafn) {
+    if (stats) return leafn ? pick_walk<true, true>(mode) : pick_walk<true, false>(mode);
+    return leafn ? pick_walk<false, true>(mode) : pick_walk<false, false>(mode);
+}
+
+// 64-bit segment indices, and leaf references that do not fit an item (leaf
+// sizes above 1 from 2^28 triangles on), stay with the general loop.
+bool walk_fits(int64_t nR, int64_t n, int leaf_size) {
+    return nR < (int64_t)1 << 31 && (leaf_size == 1 || n < (int64_t)1 << 28);
+}
+
+// First item of every segment's walk over a mesh of n triangles at offset
+// off: the Karras root's slot (not the root slot above it, whose only use is
+// the box of the whole mesh: 9.0 -> 8.0 visits per segment of the paper-scale
+// query), or the mesh as one leaf.
+int walk_start(int off, int n, int leaf_size) {
+    if (n == 0) return kNoRoot;
+    if (n > leaf_size) return off;
+    return leaf_size > 1 ? ~((off << 3) | (n - 1)) : ~off;
 }
 
 struct OccKey {
@@ -148,9 +201,17 @@ int max_block(const void* fn, int block) {
 
 cudaError_t launch_trace(const TraceParams& P, int mode, int stack, bool stats, int block,
                          int width, cudaStream_t s) {
-    KernelFn fn = trace_kernel(mode, stack, stats, width, P.root < 0);
+    // The phased loop (walk.cuh) serves what the default options ask for.  The
+    // general loop keeps the options that it has no code for: a smaller stack,
+    // 4-wide nodes, a treelet.
+    const bool leafn = P.leaf_size > 1;
+    const bool walk = stack == 64 && width == 2 && P.root >= 0 &&
+                      walk_fits(P.nR, P.nT, P.leaf_size);
+    KernelFn fn = walk ? walk_kernel(mode, stats, leafn)
+                       : trace_kernel(mode, stack, stats, width, P.root < 0);
     block = max_block((const void*)fn, block);  // register-limited kernels cap the block
-    const int smem = P.smem_nodes > 0 ? P.smem_nodes * 64 : 0;
+    const int smem = walk ? (block / 32) * (int)sizeof(WalkStage)
+                          : P.smem_nodes > 0 ? P.smem_nodes * 64 : 0;
     int grid = 0;
     cudaError_t e = occupancy_grid((const void*)fn, block, smem, &grid);
     if (e != cudaSuccess) return e;
@@ -161,6 +222,7 @@ cudaError_t launch_trace(const TraceParams& P, int mode, int stack, bool stats, 
     f = f < kFetchMin ? kFetchMin : f > kFetchChunk ? kFetchChunk : f / 32 * 32;
     TraceParams Q = P;
     Q.fetch = (int)f;
+    if (walk) Q.root = walk_start(0, P.nT, P.leaf_size);
     const int64_t warps_needed = (P.nR + f - 1) / f;
     const int64_t blocks_needed = (warps_needed + block / 32 - 1) / (block / 32);
     if (blocks_needed < grid) grid = (int)blocks_needed;
