@@ -55,8 +55,10 @@ size_t carve(TreeBufs& tb, int64_t N, int M, int nblk, char* base) {
     tb.vals[1] = (uint32_t*)take(4 * n1);
     tb.hist = (uint32_t*)take(4 * (size_t)rsi::kSortBins * (tb.ntiles > 0 ? tb.ntiles : 1));
     tb.totals = (uint32_t*)take(4 * (size_t)rsi::kSortBins);
-    tb.partial = (float*)take(4 * 6 * (size_t)(nblk > 0 ? nblk : 1));
+    tb.partial = (float*)take(4 * 12 * (size_t)(nblk > 0 ? nblk : 1));
     tb.bounds = (float*)take(4 * 6 * (size_t)M);
+    tb.frame = (float4*)take(16 * 2 * (size_t)M);
+    tb.coarse = (int32_t*)take(4 * (size_t)M);
     tb.rootbox = (float4*)take(16 * 2 * (size_t)M);
     tb.child = (int32_t*)take(4 * 2 * n1);
     tb.range = (int32_t*)take(4 * 2 * n1);
@@ -67,9 +69,13 @@ size_t carve(TreeBufs& tb, int64_t N, int M, int nblk, char* base) {
     tb.nbox = (float4*)take(16 * 2 * n1);
     tb.lbox = (float4*)take(16 * 2 * n1);
     tb.nodes = (float4*)take(16 * 4 * n1);
+    tb.qnodes = (float4*)take(16 * 4 * n1);
+    tb.par = (int32_t*)take(4 * n1);
     tb.nodes4 = (float4*)take(16 * 8 * n1);
-    tb.tris = (float4*)take(16 * 3 * n1);
+    tb.tris = (float4*)take(16 * 3 * (n1 + 1));
     tb.treelet = (float4*)take(M == 1 ? 16 * 4 * (size_t)rsi::kTreeletMax : 16);
+    // cleared when the handle is made with the scratch words that follow the tree
+    tb.done = (int32_t*)take(4 * (size_t)M);
     tb.treelet_n = (int32_t*)take(4);
     tb.status = (int32_t*)take(4);
     return off;
@@ -174,7 +180,9 @@ struct rsi_bvh_s {
     TreeBufs tb;
     char* mem = nullptr;
     size_t bytes = 0;
-    unsigned long long* scratch = nullptr;  // [0] work counter, [1..7] stats, [8..9] streamed counters
+    unsigned long long* scratch = nullptr;  // [0] work counter, [1..7] stats, [8..9] streamed counters,
+                                            // [10..15] phased loop: counter and finished blocks of
+                                            // the main and the two pipeline streams
     bool built = false;
     bool nodes4_valid = false;  // 4-wide records built for the current tree
     // stream of the last call that queued work on the handle's memory: calls
@@ -270,7 +278,8 @@ rsi_status rsi_bvh_create(int64_t nV, int64_t nT, const rsi_build_opts* opt, rsi
     h->nT = nT;
     h->leaf = leaf;
     h->levels = levels;
-    const int nblk = (int)((nT + rsi::kBuildChunk - 1) / rsi::kBuildChunk);
+    const int chunk = rsi::bounds_chunk(nT);
+    const int nblk = (int)((nT + chunk - 1) / chunk);
     TreeBufs tb;
     memset(&tb, 0, sizeof(tb));
     size_t bytes = carve(tb, nT, 1, nblk, nullptr) + 256;
@@ -282,6 +291,7 @@ rsi_status rsi_bvh_create(int64_t nV, int64_t nT, const rsi_build_opts* opt, rsi
         return e == cudaErrorMemoryAllocation ? RSI_ERR_OOM : RSI_ERR_CUDA;
     }
     carve(tb, nT, 1, nblk, h->mem);
+    tb.chunk = chunk;
     h->scratch = (unsigned long long*)(h->mem + bytes - 256);
     tb.leaf_size = leaf;
     tb.height_axis = height;
@@ -290,8 +300,7 @@ rsi_status rsi_bvh_create(int64_t nV, int64_t nT, const rsi_build_opts* opt, rsi
     h->tb = tb;
     h->bytes = bytes;
     h->stream = cs;
-    e = cudaMemsetAsync(tb.status, 0, 4, cs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(tb.treelet_n, 0, 4, cs);
+    e = cudaMemsetAsync(tb.done, 0, (size_t)(h->mem + bytes - (char*)tb.done), cs);
     if (e != cudaSuccess) {
         cudaGetLastError();
         rsi::dev_free(h->hooks, h->mem, cs);
@@ -475,7 +484,7 @@ rsi_status rsi_bvh_export(rsi_bvh h, rsi_stream s, float* bounds, uint32_t* code
 static rsi_status intersect_impl(rsi_bvh h, const float* dA, const float* dB, int64_t nR,
                                  rsi_mode mode, const rsi_output* out, const rsi_launch_opts* lo,
                                  rsi_stream s, bool force_stats,
-                                 unsigned long long* work = nullptr,
+                                 int pipe = 0,
                                  const int32_t* ready = nullptr, int64_t ready_chunk = 1) {
     if (!h || nR < 0) return RSI_ERR_ARG;
     if (mode != RSI_MODE_BOOL && mode != RSI_MODE_COUNT && mode != RSI_MODE_NEAREST)
@@ -510,11 +519,15 @@ static rsi_status intersect_impl(rsi_bvh h, const float* dA, const float* dB, in
     P.nT = (int)h->nT;
     P.nodes = h->tb.nodes;
     P.nodes4 = h->tb.nodes4;
+    P.qnodes = h->tb.qnodes;
+    P.frame = h->tb.frame;
+    P.coarse = h->tb.coarse;
     P.tris = h->tb.tris;
     P.treelet = h->tb.treelet;
     P.treelet_n = h->tb.treelet_n;
     P.smem_nodes = c.smem_nodes;
-    P.work = work ? work : h->scratch;
+    P.work = h->scratch + (pipe ? 7 + pipe : 0);
+    P.walk_work = h->scratch + 10 + 2 * pipe;
     P.stats = h->scratch + 1;
     P.max_visits = (int)h->nT + 2;
     P.status = h->tb.status;
@@ -535,7 +548,9 @@ static rsi_status intersect_impl(rsi_bvh h, const float* dA, const float* dB, in
     }
     if (c.stats)
         RSI_CK(cudaMemsetAsync(P.stats, 0, rsi::kStatCounters * 8, (cudaStream_t)s));
-    if (c.packet)
+    // packets use the phased loop's items; meshes beyond those (walk_fits) get
+    // the same results one segment per lane
+    if (c.packet && rsi::walk_fits(1, h->nT, h->leaf))
         RSI_CK(rsi::launch_trace_packet(P, mode, c.stats, (cudaStream_t)s));
     else
         RSI_CK(rsi::launch_trace(P, mode, c.stack, c.stats, c.block, c.width, (cudaStream_t)s));
@@ -703,7 +718,7 @@ static rsi_status intersect_streamed(rsi_bvh h, const float* hA, const float* hB
     dout.flag = dflag;
     RSI_CK(cudaStreamWaitEvent(cs, h->sev_reset, 0));  // never a previous call's flags
     const rsi_status st = intersect_impl(h, dA, dB, nR, RSI_MODE_BOOL, &dout, lo, (rsi_stream)cs,
-                                         false, nullptr, ready, ch);
+                                         false, 0, ready, ch);
     if (st != RSI_OK) {
         cudaStreamWaitEvent(cs, h->pev_done[0], 0);  // hA, hB are read until then
         return st;
@@ -818,7 +833,7 @@ static rsi_status intersect_host_impl(rsi_bvh h, const float* hA, const float* h
             dout.dist = (float*)(o + o1 + 2 * o3);
         }
         st = intersect_impl(h, dA, dB, n, mode, &dout, &lo2, (rsi_stream)S, false,
-                            h->scratch + 8 + q);
+                            1 + q);
         if (st != RSI_OK) return st;
         auto back = [&](void* host, const void* dev, size_t bytes) -> cudaError_t {
             return host ? cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, S)
@@ -961,6 +976,9 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
     int nblk = 0;
     std::vector<MeshDesc> table(n);
     std::vector<int32_t> blkmesh;
+    int64_t total = 0;
+    for (int k = 0; k < n; ++k) total += items[k].nT > 0 ? items[k].nT : 0;
+    const int chunk = rsi::bounds_chunk(total);
     for (int k = 0; k < n; ++k) {
         const rsi_batch_item& it = items[k];
         if (it.nV < 0 || it.nT < 0 || it.nR < 0) return RSI_ERR_ARG;
@@ -976,7 +994,7 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         md.n = (int32_t)it.nT;
         md.off = (int32_t)N;
         md.blk0 = nblk;
-        md.nblk = (int32_t)((it.nT + rsi::kBuildChunk - 1) / rsi::kBuildChunk);
+        md.nblk = (int32_t)((it.nT + chunk - 1) / chunk);
         if (it.height_axis < 0 || it.height_axis > 3) return RSI_ERR_ARG;
         md.height_axis = it.height_axis > 0 ? it.height_axis : height;
         for (int q = 0; q < md.nblk; ++q) blkmesh.push_back(k);
@@ -1008,6 +1026,7 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         d.B = it.dB;
         d.nR = it.nR;
         d.root = it.nT > 0 ? (int)(table[k].off + it.nT - 1) : rsi::kNoRoot;
+        d.n = (int)it.nT;
         d.start = rsi::walk_start(table[k].off, (int)it.nT, leaf);
         walk = walk && rsi::walk_fits(it.nR, N, leaf);
         d.mode = it.mode;
@@ -1052,6 +1071,7 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         return e == cudaErrorMemoryAllocation ? RSI_ERR_OOM : RSI_ERR_CUDA;
     }
     carve(tb, N, n, nblk, b->mem);
+    tb.chunk = chunk;
     tb.leaf_size = leaf;
     tb.height_axis = height;
     tb.top_levels = 0;
@@ -1074,6 +1094,7 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         e = cudaMemcpyAsync(b->d_tiles, tiles.data(), sizeof(rsi::BatchTile) * tiles.size(),
                             cudaMemcpyHostToDevice, cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(tb.status, 0, 4, cs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tb.done, 0, 4 * (size_t)n, cs);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cs);  // host tables go out of scope
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork.start, cudaEventDisableTiming);
@@ -1126,6 +1147,9 @@ rsi_status rsi_batch_intersect(rsi_batch b, rsi_stream s) {
     P.n_tiles = b->n_tiles;
     P.nodes = b->tb.nodes;
     P.nodes4 = b->tb.nodes4;
+    P.qnodes = b->tb.qnodes;
+    P.frame = b->tb.frame;
+    P.coarse = b->tb.coarse;
     P.tris = b->tb.tris;
     P.work = b->work;
     P.max_visits = b->tb.N + 2;

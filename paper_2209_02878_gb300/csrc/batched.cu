@@ -80,6 +80,7 @@ __global__ void __maxnreg__(kWalkRegs) k_batch_walk(BatchParams P) {
     const int lane = threadIdx.x & 31;
     TraceCtx C;
     C.nodes = P.nodes;
+    C.qnodes = P.qnodes;
     C.tris = P.tris;
     C.max_visits = P.max_visits;
     C.fetch = kFetchChunk;  // unused: each tile is one warp's whole pool
@@ -99,6 +100,8 @@ __global__ void __maxnreg__(kWalkRegs) k_batch_walk(BatchParams P) {
         C.B = it.B;
         C.nR = it.nR;
         C.out = it.out;
+        C.frame = P.frame + 2 * tile.item;
+        C.coarse = it.n > 0 && walk_coarse(P.coarse[tile.item], it.n);
         walk_loop<MODE, false, LEAFN>(C, sg, it.start, nullptr, tile.lo, tile.hi, st, segs);
     }
 }
@@ -112,9 +115,10 @@ static BatchFn batch_walk_kernel(int mode, bool leafn) {
     return leafn ? k_batch_walk<RSI_MODE_NEAREST, true> : k_batch_walk<RSI_MODE_NEAREST, false>;
 }
 
-// Zero the compaction counters of the items that compact.
-__global__ void k_zero_counts(const BatchItemDev* items, int n) {
+// Zero the work counters and the compaction counters of the items that compact.
+__global__ void k_zero_counts(const BatchItemDev* items, int n, unsigned long long* work) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < 3) work[k] = 0ull;
     if (k < n && items[k].out.hit_idx) *items[k].out.n_hits = 0;
 }
 
@@ -170,9 +174,9 @@ static cudaError_t launch_batch_walk(const BatchParams& P, int block, cudaStream
 cudaError_t launch_batch(const BatchParams& P, int block, int stack, cudaStream_t s,
                          const BatchFork& fk) {
     if (P.n_tiles == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(P.work, 0, 3 * sizeof(unsigned long long), s);
+    k_zero_counts<<<(P.n_items + 255) / 256, 256, 0, s>>>(P.items, P.n_items, P.work);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_zero_counts<<<(P.n_items + 255) / 256, 256, 0, s>>>(P.items, P.n_items);
     if (P.walk && stack == 64) return launch_batch_walk(P, block, s, fk);
     const void* fn = batch_kernel(stack);
     block = max_block(fn, block);

@@ -68,50 +68,114 @@ __device__ __forceinline__ int block_mesh(const MeshArgs& ma, int b) {
     return ma.M == 1 ? 0 : ma.blk_mesh[b];
 }
 
-// Block-wide min / max of 6 values (lo xyz, hi xyz); result valid in thread 0.
-__device__ __forceinline__ void block_minmax6(float v[6]) {
-    __shared__ float red[6][kBuildThreads / 32];
+// Block-wide min / max of the N values (each run of six: lo xyz, hi xyz);
+// result valid in thread 0.
+template <int N>
+__device__ __forceinline__ void block_minmax(float v[N]) {
+    __shared__ float red[N][kBuildThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < N; ++k) {
         float x = v[k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float y = __shfl_xor_sync(0xffffffffu, x, o);
-            x = k < 3 ? fminf(x, y) : fmaxf(x, y);
+            x = k % 6 < 3 ? fminf(x, y) : fmaxf(x, y);
         }
         if (lane == 0) red[k][w] = x;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
+        for (int k = 0; k < N; ++k) {
             float x = red[k][0];
             for (int q = 1; q < kBuildThreads / 32; ++q)
-                x = k < 3 ? fminf(x, red[k][q]) : fmaxf(x, red[k][q]);
+                x = k % 6 < 3 ? fminf(x, red[k][q]) : fmaxf(x, red[k][q]);
             v[k] = x;
         }
     }
 }
 
-// a1: per-block support interval of the (finite) centroids.
-__global__ void __launch_bounds__(kBuildThreads) k_bounds(MeshArgs ma, TreeBufs tb) {
+// Grid of the four-way nodes over the vertex box (lo, hi): X = 1 + (x - o) s.
+// The scale leaves 8 of the 32,768 steps free for the rounding outward; an
+// axis far thinner than the widest one gets a 2^20th of that one's extent.
+// Without a valid triangle (lo > hi) any grid does: every box is empty.
+__device__ __forceinline__ void write_frame(const TreeBufs& tb, int m, const float* lo,
+                                            const float* hi) {
+    float o[3] = {0.f, 0.f, 0.f}, s[3] = {1.f, 1.f, 1.f};
+    if (lo[0] <= hi[0]) {
+        float e[3], widest = 0x1p-80f;
+        for (int k = 0; k < 3; ++k) {
+            e[k] = __fsub_rn(hi[k], lo[k]);
+            widest = fmaxf(widest, e[k]);
+        }
+        for (int k = 0; k < 3; ++k) {
+            o[k] = lo[k];
+            s[k] = __fdiv_rn(32760.f / 32768.f, fmaxf(e[k], widest * 0x1p-20f));
+        }
+    }
+    tb.frame[2 * m] = make_float4(o[0], o[1], o[2], 0.f);
+    tb.frame[2 * m + 1] = make_float4(s[0], s[1], s[2], 0.f);
+}
+
+// a1: support interval of the (finite) centroids and of the vertices of the
+// valid triangles, per mesh: per block, then over the blocks by the mesh's
+// last block to finish.  A refit keeps the build's centroid interval.
+// (Reducing all blocks' partials again in every block of k_morton took that
+// kernel 42 us at 1.31M triangles.)
+__global__ void __launch_bounds__(kBuildThreads) k_bounds(MeshArgs ma, TreeBufs tb, int refit) {
+    __shared__ int last;
     const int b = blockIdx.x;
-    const MeshDesc md = mesh_of(ma, block_mesh(ma, b));
-    const int j0 = (b - md.blk0) * kBuildChunk;
-    const int j1 = min(md.n, j0 + kBuildChunk);
-    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+    const int m = block_mesh(ma, b);
+    const MeshDesc md = mesh_of(ma, m);
+    const int j0 = (b - md.blk0) * tb.chunk;
+    const int j1 = (int)min((int64_t)md.n, (int64_t)j0 + tb.chunk);
+    float v[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = k % 6 < 3 ? INFINITY : -INFINITY;
+#pragma unroll 4
+    for (int j = j0 + threadIdx.x; j < j1; j += kBuildThreads) {
         float3 a, bb, c;
         if (!tri_vertices(md, j, tb.status, a, bb, c)) continue;
+        v[6] = fminf(v[6], fminf(fminf(a.x, bb.x), c.x));
+        v[7] = fminf(v[7], fminf(fminf(a.y, bb.y), c.y));
+        v[8] = fminf(v[8], fminf(fminf(a.z, bb.z), c.z));
+        v[9] = fmaxf(v[9], fmaxf(fmaxf(a.x, bb.x), c.x));
+        v[10] = fmaxf(v[10], fmaxf(fmaxf(a.y, bb.y), c.y));
+        v[11] = fmaxf(v[11], fmaxf(fmaxf(a.z, bb.z), c.z));
         const float3 ce = centroid(a, bb, c);
         if (!finite3(ce.x, ce.y, ce.z)) continue;
         v[0] = fminf(v[0], ce.x); v[1] = fminf(v[1], ce.y); v[2] = fminf(v[2], ce.z);
         v[3] = fmaxf(v[3], ce.x); v[4] = fmaxf(v[4], ce.y); v[5] = fmaxf(v[5], ce.z);
     }
-    block_minmax6(v);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 6; ++k) tb.partial[6 * b + k] = v[k];
+    block_minmax<12>(v);
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < 12; ++k) __stcg(tb.partial + 12 * (int64_t)b + k, v[k]);
+        __threadfence();
+        last = atomicAdd(tb.done + m, 1) == md.nblk - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = k % 6 < 3 ? INFINITY : -INFINITY;
+    for (int q = threadIdx.x; q < md.nblk; q += kBuildThreads) {
+        const float* p = tb.partial + 12 * (int64_t)(md.blk0 + q);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const float x = __ldcg(p + k);
+            v[k] = k % 6 < 3 ? fminf(v[k], x) : fmaxf(v[k], x);
+        }
+    }
+    __syncthreads();  // the block reduction's shared memory is used again
+    block_minmax<12>(v);
+    if (threadIdx.x == 0) {
+        if (!refit)
+            for (int k = 0; k < 6; ++k) tb.bounds[6 * m + k] = v[k];
+        write_frame(tb, m, v + 6, v + 9);
+        tb.coarse[m] = 0;
+        tb.done[m] = 0;
+    }
 }
 
 // 10-bit value -> bits at positions 3k (k = 0..9).
@@ -146,46 +210,48 @@ __device__ __forceinline__ uint32_t spread2(uint32_t x) {
     return x;
 }
 
-// a2: mesh interval from the partials, quantisation, Morton code, sort key.
+// a2: quantisation over the mesh interval, Morton code, sort key; one thread
+// per triangle of the concatenated meshes.
 __global__ void __launch_bounds__(kBuildThreads) k_morton(MeshArgs ma, TreeBufs tb) {
-    const int b = blockIdx.x;
-    const int m = block_mesh(ma, b);
-    const MeshDesc md = mesh_of(ma, m);
-    float v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    for (int q = threadIdx.x; q < md.nblk; q += blockDim.x) {
-        const float* p = tb.partial + 6 * (md.blk0 + q);
-        v[0] = fminf(v[0], p[0]); v[1] = fminf(v[1], p[1]); v[2] = fminf(v[2], p[2]);
-        v[3] = fmaxf(v[3], p[3]); v[4] = fmaxf(v[4], p[4]); v[5] = fmaxf(v[5], p[5]);
+    const int g = blockIdx.x * kBuildThreads + threadIdx.x;
+    if (g >= tb.N) return;
+    int m = 0;
+    if (ma.M > 1) {  // the mesh that holds g: the last one with off <= g and triangles
+        int hi = ma.M - 1;
+        while (m < hi) {
+            const int mid = (m + hi + 1) >> 1;
+            if (ma.table[mid].off <= g)
+                m = mid;
+            else
+                hi = mid - 1;
+        }
     }
-    block_minmax6(v);
-    __shared__ float bnd[6];
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 6; ++k) bnd[k] = v[k];
-    __syncthreads();
-    if (b == md.blk0 && threadIdx.x < 6) tb.bounds[6 * m + threadIdx.x] = bnd[threadIdx.x];
-    const int j0 = (b - md.blk0) * kBuildChunk;
-    const int j1 = min(md.n, j0 + kBuildChunk);
-    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-        float3 a, bb, c;
-        uint32_t code = 0;
-        if (tri_vertices(md, j, tb.status, a, bb, c)) {
-            const float3 ce = centroid(a, bb, c);
-            if (finite3(ce.x, ce.y, ce.z)) {
-                if (md.height_axis == 0) {
-                    code = (spread3(quant(ce.x, bnd[0], bnd[3], 1024.f)) << 2) |
-                           (spread3(quant(ce.y, bnd[1], bnd[4], 1024.f)) << 1) |
-                           spread3(quant(ce.z, bnd[2], bnd[5], 1024.f));
-                } else {  // height field: the other two axes, the first one high
-                    const float cc[3] = {ce.x, ce.y, ce.z};
-                    const int a = md.height_axis == 1 ? 1 : 0, b = md.height_axis == 3 ? 1 : 2;
-                    code = (spread2(quant(cc[a], bnd[a], bnd[3 + a], 32768.f)) << 1) |
-                           spread2(quant(cc[b], bnd[b], bnd[3 + b], 32768.f));
-                }
+    const MeshDesc md = mesh_of(ma, m);
+    const int j = g - md.off;
+    float bnd[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) bnd[k] = tb.bounds[6 * m + k];
+    float3 a, bb, c;
+    uint32_t code = 0;
+    if (tri_vertices(md, j, tb.status, a, bb, c)) {
+        const float3 ce = centroid(a, bb, c);
+        if (finite3(ce.x, ce.y, ce.z)) {
+            if (md.height_axis == 0) {
+                code = (spread3(quant(ce.x, bnd[0], bnd[3], 1024.f)) << 2) |
+                       (spread3(quant(ce.y, bnd[1], bnd[4], 1024.f)) << 1) |
+                       spread3(quant(ce.z, bnd[2], bnd[5], 1024.f));
+            } else {  // height field: the other two axes, the first one high
+                const bool ax = md.height_axis == 1, az = md.height_axis == 3;
+                const uint32_t q0 = ax ? quant(ce.y, bnd[1], bnd[4], 32768.f)
+                                       : quant(ce.x, bnd[0], bnd[3], 32768.f);
+                const uint32_t q1 = az ? quant(ce.y, bnd[1], bnd[4], 32768.f)
+                                       : quant(ce.z, bnd[2], bnd[5], 32768.f);
+                code = (spread2(q0) << 1) | spread2(q1);
             }
         }
-        tb.keys[0][md.off + j] = ((uint64_t)m << 32) | code;
-        tb.vals[0][md.off + j] = (uint32_t)(md.off + j);
     }
+    tb.keys[0][g] = ((uint64_t)m << 32) | code;
+    tb.vals[0][g] = (uint32_t)g;
 }
 
 // ---------------------------------------------------------------- a4
@@ -227,6 +293,8 @@ __global__ void k_karras(MeshArgs ma, TreeBufs tb, const uint64_t* __restrict__ 
     const int right = (hi == gam + 1) ? -(off + gam + 2) : off + gam + 1;
     tb.child[2 * g] = left;
     tb.child[2 * g + 1] = right;
+    if (left >= 0) tb.par[left] = 2 * g;
+    if (right >= 0) tb.par[right] = 2 * g + 1;
     tb.range[2 * g] = off + lo;
     tb.range[2 * g + 1] = off + hi;
 }
@@ -258,6 +326,49 @@ __device__ __forceinline__ void write_node(float4* nodes, int slot, float4 l0, f
     __stcg(o + 1, make_float4(f[2], f[8], f[3], f[9]));
     __stcg(o + 2, make_float4(f[4], f[10], f[5], f[11]));
     __stcg(o + 3, make_float4(f[12], f[13], f[14], f[15]));
+}
+
+// One axis of a child box on the grid, rounded outward: lo | hi << 16, each with
+// bit 15 set.  (x - o) s carries two roundings, below 2^-8 of a step, so the
+// 1/16 step leaves the grid box around the exact one; an empty box becomes
+// lo = 32767, hi = 0, which no segment enters.
+__device__ __forceinline__ uint32_t grid_axis(float lo, float hi, float o, float s) {
+    if (lo > hi) return 0x8000ffffu;
+    const float a = __fmul_rn(__fmul_rn(__fsub_rn(lo, o), s), 32768.f);
+    const float b = __fmul_rn(__fmul_rn(__fsub_rn(hi, o), s), 32768.f);
+    const uint32_t q0 = (uint32_t)fminf(fmaxf(floorf(a - 0.0625f), 0.f), 32767.f);
+    const uint32_t q1 = (uint32_t)fmaxf(fminf(ceilf(b + 0.0625f), 32767.f), 0.f);
+    return (0x8000u | q0) | (0x8000u | q1) << 16;
+}
+
+// Half `h` of qnodes: boxes and items of two siblings.
+__device__ __forceinline__ void write_half(const TreeBufs& tb, int m, int h, float4 l0, float4 h0,
+                                           int x0, float4 l1, float4 h1, int x1) {
+    const float4 o = tb.frame[2 * m], s = tb.frame[2 * m + 1];
+    uint4* q = (uint4*)(tb.qnodes + 2 * (int64_t)h);
+    __stcg(q, make_uint4(grid_axis(l0.x, h0.x, o.x, s.x), grid_axis(l0.y, h0.y, o.y, s.y),
+                         grid_axis(l0.z, h0.z, o.z, s.z), grid_axis(l1.x, h1.x, o.x, s.x)));
+    __stcg(q + 1, make_uint4(grid_axis(l1.y, h1.y, o.y, s.y), grid_axis(l1.z, h1.z, o.z, s.z),
+                             (uint32_t)x0, (uint32_t)x1));
+}
+
+__device__ __forceinline__ int leaf_item(const TreeBufs& tb, int pos, int cnt) {
+    return ~(tb.leaf_size > 1 ? pos << 3 | (cnt - 1) : pos);
+}
+
+// What internal slot `slot` writes of qnodes: its own half of its parent's
+// record (the Karras root has none; a slot collapsed into a leaf is not
+// reached), and the halves of its own record that stand for a leaf child.
+__device__ __forceinline__ void write_qnode(const TreeBufs& tb, int m, int slot, bool root,
+                                            float4 l0, float4 h0, int ref0, int cnt0, float4 l1,
+                                            float4 h1, int ref1, int cnt1) {
+    const int x0 = cnt0 > 0 ? leaf_item(tb, ref0, cnt0) : ref0;
+    const int x1 = cnt1 > 0 ? leaf_item(tb, ref1, cnt1) : ref1;
+    if (!root) write_half(tb, m, tb.par[slot], l0, h0, x0, l1, h1, x1);
+    const float4 e0 = make_float4(1.f, 1.f, 1.f, 0.f), e1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int none = leaf_item(tb, tb.N, 1);
+    if (cnt0 > 0) write_half(tb, m, 2 * slot, l0, h0, x0, e0, e1, none);
+    if (cnt1 > 0) write_half(tb, m, 2 * slot + 1, l1, h1, x1, e0, e1, none);
 }
 
 __device__ __forceinline__ void write_root(float4* nodes, int slot, float4 lo, float4 hi, int ref,
@@ -347,6 +458,9 @@ __device__ __forceinline__ void finish_node(const TreeBufs& tb, const MeshDesc& 
     __stcg(tb.nbox + 2 * (int64_t)node, f4(ul));
     __stcg(tb.nbox + 2 * (int64_t)node + 1, f4(uh));
     write_node(tb.nodes, node, f4(l0), f4(h0), ref0, cnt0, f4(l1), f4(h1), ref1, cnt1);
+    if (z0 + z1 > L)  // else collapsed into a leaf
+        write_qnode(tb, m, node, node == md.off, f4(l0), f4(h0), ref0, cnt0, f4(l1), f4(h1), ref1,
+                    cnt1);
     if (node == md.off) {  // Karras root: fill the root slot
         const int root_slot = md.off + md.n - 1;
         tb.rootbox[2 * m] = f4(ul);
@@ -398,11 +512,13 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
     int2* srg = sch + kBoxBlock;               // leaf ranges of slots base ..
     const int tid = threadIdx.x, lane = tid & 31;
     const int base = blockIdx.x * kBoxBlock, g = base + tid, N = tb.N;
+    if (g < 3) tb.tris[3 * (int64_t)N + g] = make_float4(0.f, 0.f, 0.f, i2f(-1));
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     MeshDesc md;
     md.off = 0;
     md.n = 0;
     int m = 0;
+    bool coarse = false;  // a leaf box that the four-way nodes' grid blurs
     if (g < N) {
         m = (int)(keys[g] >> 32);
         md = mesh_of(ma, m);
@@ -425,6 +541,12 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
         }
         __stcg(tb.lbox + 2 * (int64_t)g, f4(lo));
         __stcg(tb.lbox + 2 * (int64_t)g + 1, f4(hi));
+        if (ok) {
+            const float4 s = tb.frame[2 * m + 1];
+            const float e = fmaxf(fmaxf((hi[0] - lo[0]) * s.x, (hi[1] - lo[1]) * s.y),
+                                  (hi[2] - lo[2]) * s.z);
+            coarse = e * 32768.f < kCoarseSteps;
+        }
         if (md.n == 1) {
             write_root(tb.nodes, md.off, f4(lo), f4(hi), g, 1);
             tb.rootbox[2 * m] = f4(lo);
@@ -435,6 +557,13 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
     for (int c = 0; c < 3; ++c) {
         st[c * kStEntries + tid] = lo[c];
         st[(3 + c) * kStEntries + tid] = hi[c];
+    }
+    {  // one atomic per warp and mesh
+        const unsigned cb = __ballot_sync(0xffffffffu, coarse);
+        if (cb) {
+            const unsigned peers = __match_any_sync(0xffffffffu, m) & cb;
+            if (coarse && lane == __ffs(peers) - 1) atomicAdd(tb.coarse + m, __popc(peers));
+        }
     }
     // slots whose range crosses a block boundary, for the second pass
     const bool inner = g < N && g - md.off < md.n - 1;  // an internal slot, not a root slot
@@ -741,9 +870,9 @@ cudaError_t build_prepare() {
 cudaError_t build_tree(TreeBufs& tb, const MeshArgs& ma, cudaStream_t s, bool refit) {
     const int N = tb.N;
     if (N == 0) return cudaSuccess;
+    k_bounds<<<tb.nblk, kBuildThreads, 0, s>>>(ma, tb, refit ? 1 : 0);
     if (!refit) {
-        k_bounds<<<tb.nblk, kBuildThreads, 0, s>>>(ma, tb);
-        k_morton<<<tb.nblk, kBuildThreads, 0, s>>>(ma, tb);
+        k_morton<<<cdiv(N, kBuildThreads), kBuildThreads, 0, s>>>(ma, tb);
         int shifts[8], np = 0;
         for (int sh = 0; sh < 32; sh += 8) shifts[np++] = sh;
         for (int sh = 32; sh < 64 && ((int64_t)(tb.M - 1) >> (sh - 32)) > 0; sh += 8)

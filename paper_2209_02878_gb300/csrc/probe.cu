@@ -104,6 +104,7 @@ extern "C" rsi_status rsi_selftest_stream_wait(int32_t polls, int64_t nR, rsi_st
         P.ready_chunk = chunk;
         P.wait_polls = polls;
         P.work = (unsigned long long*)(mem + seg_b + flag_b + ready_b);
+        P.walk_work = P.work + 1;
         P.status = (int32_t*)(mem + seg_b + flag_b + ready_b + 128);
         P.max_visits = 2;
         if (cudaEventRecord(e0, cs) != cudaSuccess ||

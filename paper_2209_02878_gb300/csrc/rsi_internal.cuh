@@ -31,7 +31,21 @@
 //                    {lo.x[4]} {lo.y[4]} {lo.z[4]} {hi.x[4]} {hi.y[4]}
 //                    {hi.z[4]} {ref[4]} {cnt[4]}; traversal over these visits
 //                    every other level of the binary tree
-//   tris[3N]         triangles in leaf order: {v0, orig id}, {v1, -}, {v2, -}
+//   qnodes[4N]       for the phased traversal: the boxes of the slot's (up to)
+//                    four grandchildren on a 15-bit grid over the mesh's box,
+//                    64 B in two halves, one per child: per grandchild and
+//                    axis one word (0x8000 | lo) | (0x8000 | hi) << 16, x y z
+//                    of the first, x y z of the second, then their two items
+//                    (slot >= 0; leaf ~position, or ~(8 position + count - 1)
+//                    when leaf_size > 1).  A half is written by the child
+//                    itself (par); where the child is a leaf, by the slot, as
+//                    {leaf, empty box with the null triangle as its leaf}
+//   par[N]           2 * parent slot + side of an internal slot
+//   frame[2M]        the grid of each mesh: origin o and scale s per axis, a
+//                    coordinate x at X = 1 + (x - o) s in [1, 2); grid step
+//                    2^-15 in X
+//   tris[3N + 3]     triangles in leaf order: {v0, orig id}, {v1, -}, {v2, -};
+//                    then the null triangle (zero edges: never hit)
 //   treelet[4 S]     breadth-first copy of the top of one mesh's tree
 #pragma once
 
@@ -50,7 +64,7 @@ constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys per tile
 constexpr int kSortTileMin = kSortThreads * 4;         // 1024 keys per tile (small sorts)
 constexpr int kSortBins = 256;
 constexpr int kBuildThreads = 256;
-constexpr int kBuildChunk = 512;    // triangles per block in bounds / Morton
+constexpr float kCoarseSteps = 8.f;  // a leaf box below this many grid steps is coarse
 constexpr int kBoxBlock = 512;      // sorted leaves per block of the bottom-up box pass
 
 // FP32 filter constants (see mt32 below).
@@ -61,13 +75,17 @@ constexpr float kRangeHi = 0x1p30f;
 constexpr float kSlabSlack = 0x1p-18f;
 constexpr float kTinyDir = 0x1p-60f;
 
+// Triangles per block of the bounds pass: enough blocks for a small mesh, few
+// enough partials for the last block of a large one.
+inline int bounds_chunk(int64_t n) { return n <= (int64_t)1 << 18 ? 512 : 2048; }
+
 struct MeshDesc {
     const float* V;
     const int32_t* T;
     int64_t nV;
     int32_t n;     // triangles
     int32_t off;   // offset in concatenated triangle / node arrays
-    int32_t blk0;  // first block of this mesh in the bounds / Morton grid
+    int32_t blk0;  // first block of this mesh in the bounds grid
     int32_t nblk;
     int32_t height_axis;  // Morton code: 0 over x, y, z; 1..3 that axis left out
 };
@@ -91,9 +109,13 @@ struct TreeBufs {
     uint32_t* hist;
     uint32_t* totals;  // kSortBins digit totals of the current sort pass
     int32_t ntiles;
-    int32_t nblk;     // blocks of the bounds / Morton grid
-    float* partial;   // 6 * nblk
+    int32_t nblk;     // blocks of the bounds grid
+    int32_t chunk;    // triangles per block of it (bounds_chunk)
+    float* partial;   // 12 * nblk: centroid and vertex intervals per block
     float* bounds;    // 6 * M
+    float4* frame;    // 2 * M: grid of qnodes {origin, -}, {scale, -}
+    int32_t* coarse;  // M: leaves whose box spans fewer than kCoarseSteps grid steps
+    int32_t* done;    // M: blocks of the mesh that k_bounds has finished (0 between launches)
     float4* rootbox;  // 2 * M: box of each mesh (lo, hi)
     int32_t* child;   // 2N
     int32_t* range;   // 2N
@@ -105,8 +127,10 @@ struct TreeBufs {
     float4* nbox;     // 2N
     float4* lbox;     // 2N
     float4* nodes;    // 4N
+    float4* qnodes;   // 4N: 64-byte records of the phased traversal
+    int32_t* par;     // N: where an internal slot's half lies in qnodes
     float4* nodes4;   // 8N: 4-wide records (grandchildren of each slot)
-    float4* tris;     // 3N
+    float4* tris;     // 3N + 3
     float4* treelet;  // 4 * kTreeletMax (single-mesh trees)
     int32_t* treelet_n;
     int32_t* status;  // device status word (rsi_status)

@@ -29,11 +29,17 @@ struct TraceParams {
     int nT;         // triangles
     const float4* nodes;
     const float4* nodes4;
+    const float4* qnodes;  // phased loop: four-way records, their grid, and the
+    const float4* frame;   // number of leaves the grid is too coarse for
+    const int32_t* coarse;
     const float4* tris;
     const float4* treelet;
     const int32_t* treelet_n;
     int smem_nodes;
-    unsigned long long* work;   // zeroed before each launch
+    unsigned long long* work;   // general loop: zeroed before each launch
+    // phased loop: work counter and finished blocks, both 0 between launches
+    // (the last block to finish clears them)
+    unsigned long long* walk_work;
     unsigned long long* stats;  // 6 counters (STATS launches)
     int max_visits;             // node fetches per segment before giving up
     int fetch;                  // segments per warp fetch (set by launch_trace)
@@ -45,7 +51,7 @@ struct TraceParams {
     TravOut out;
 };
 
-// Enqueue one traversal (2 memsets + 1 kernel).
+// Enqueue one traversal.
 cudaError_t launch_trace(const TraceParams& P, int mode, int stack, bool stats, int block,
                          int width, cudaStream_t s);
 
@@ -90,6 +96,7 @@ struct BatchItemDev {
     int64_t nR;
     int root;   // root slot of the item's mesh, or kNoRoot
     int start;  // first item of the phased loop (walk_start)
+    int n;      // triangles of the item's mesh
     int mode;
     TravOut out;
 };
@@ -109,6 +116,9 @@ struct BatchParams {
     int64_t n_tiles;
     const float4* nodes;
     const float4* nodes4;
+    const float4* qnodes;   // as in TraceParams, frame and coarse per item
+    const float4* frame;
+    const int32_t* coarse;
     const float4* tris;
     unsigned long long* work;
     int max_visits;
@@ -124,6 +134,9 @@ struct BatchFork {
     cudaStream_t aux[2];
     cudaEvent_t start, done[2];
 };
+
+using WalkFn = void (*)(TraceParams);
+WalkFn walk_kernel(int mode, bool stats, bool leafn, bool small);
 
 // Whether the phased loop (walk.cuh) can take nR segments against trees of n
 // triangles in all, and its first item for a mesh of n triangles at off.

@@ -88,58 +88,6 @@ KernelFn trace_kernel(int mode, int stack, bool stats, int width, bool treelet) 
     return stats ? pick_mode<true, 2, false>(mode, stack) : pick_mode<false, 2, false>(mode, stack);
 }
 
-template <int MODE, bool STATS, bool LEAFN>
-__global__ void __maxnreg__(kWalkRegs) k_walk(TraceParams P) {
-    extern __shared__ float4 stage4[];
-    TraceCtx C;
-    C.A = P.A;
-    C.B = P.B;
-    C.nR = P.nR;
-    C.nodes = P.nodes;
-    C.tris = P.tris;
-    C.max_visits = P.max_visits;
-    C.fetch = P.fetch;
-    C.ready = P.ready;
-    C.ready_chunk = P.ready_chunk;
-    C.wait_polls = P.wait_polls > 0 ? P.wait_polls : kWaitPolls;
-    C.order = P.order;
-    C.status = P.status;
-    C.out = P.out;
-    TravStats st = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
-    unsigned long long segs = 0;
-    WalkStage& sg = ((WalkStage*)stage4)[threadIdx.x >> 5];
-    walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, P.work, 0, P.nR, st, segs);
-    if (STATS) flush_stats(st, P.stats, segs);
-}
-
-template <bool STATS, bool LEAFN>
-static KernelFn pick_walk(int mode) {
-    if (mode == RSI_MODE_BOOL) return k_walk<RSI_MODE_BOOL, STATS, LEAFN>;
-    if (mode == RSI_MODE_COUNT) return k_walk<RSI_MODE_COUNT, STATS, LEAFN>;
-    return k_walk<RSI_MODE_NEAREST, STATS, LEAFN>;
-}
-
-static KernelFn walk_kernel(int mode, bool stats, bool leafn) {
-    if (stats) return leafn ? pick_walk<true, true>(mode) : pick_walk<true, false>(mode);
-    return leafn ? pick_walk<false, true>(mode) : pick_walk<false, false>(mode);
-}
-
-// 64-bit segment indices, and leaf references that do not fit an item (leaf
-// sizes above 1 from 2^28 triangles on), stay with the general loop.
-bool walk_fits(int64_t nR, int64_t n, int leaf_size) {
-    return nR < (int64_t)1 << 31 && (leaf_size == 1 || n < (int64_t)1 << 28);
-}
-
-// First item of every segment's walk over a mesh of n triangles at offset
-// off: the Karras root's slot (not the root slot above it, whose only use is
-// the box of the whole mesh: 9.0 -> 8.0 visits per segment of the paper-scale
-// query), or the mesh as one leaf.
-int walk_start(int off, int n, int leaf_size) {
-    if (n == 0) return kNoRoot;
-    if (n > leaf_size) return off;
-    return leaf_size > 1 ? ~((off << 3) | (n - 1)) : ~off;
-}
-
 struct OccKey {
     const void* fn;
     int block, smem, dev;
@@ -207,28 +155,42 @@ cudaError_t launch_trace(const TraceParams& P, int mode, int stack, bool stats, 
     const bool leafn = P.leaf_size > 1;
     const bool walk = stack == 64 && width == 2 && P.root >= 0 &&
                       walk_fits(P.nR, P.nT, P.leaf_size);
-    KernelFn fn = walk ? walk_kernel(mode, stats, leafn)
+    KernelFn fn = walk ? walk_kernel(mode, stats, leafn, false)
                        : trace_kernel(mode, stack, stats, width, P.root < 0);
+    const int block0 = block;
     block = max_block((const void*)fn, block);  // register-limited kernels cap the block
-    const int smem = walk ? (block / 32) * (int)sizeof(WalkStage)
-                          : P.smem_nodes > 0 ? P.smem_nodes * 64 : 0;
+    int smem = walk ? (block / 32) * (int)sizeof(WalkStage)
+                    : P.smem_nodes > 0 ? P.smem_nodes * 64 : 0;
     int grid = 0;
     cudaError_t e = occupancy_grid((const void*)fn, block, smem, &grid);
     if (e != cudaSuccess) return e;
     // chunk size: about four chunks per resident warp, a multiple of 32 in
     // [kFetchMin, kFetchChunk]
-    const int64_t warps = (int64_t)grid * (block / 32);
+    int64_t warps = (int64_t)grid * (block / 32);
     int64_t f = P.nR / (4 * warps);
     f = f < kFetchMin ? kFetchMin : f > kFetchChunk ? kFetchChunk : f / 32 * 32;
     TraceParams Q = P;
+    // a segment per resident lane or less: the small launch's kernel (walk.cu;
+    // 100,003 segments over 1.31M triangles, the upper end, 194 -> 191 us)
+    if (walk && !stats && !P.ready && P.nR <= 32 * warps) {
+        fn = walk_kernel(mode, false, leafn, true);
+        block = max_block((const void*)fn, block0);
+        smem = (block / 32) * (int)sizeof(WalkStage);
+        e = occupancy_grid((const void*)fn, block, smem, &grid);
+        if (e != cudaSuccess) return e;
+        warps = (int64_t)grid * (block / 32);
+        f = (P.nR + warps - 1) / warps;
+    }
     Q.fetch = (int)f;
     if (walk) Q.root = walk_start(0, P.nT, P.leaf_size);
     const int64_t warps_needed = (P.nR + f - 1) / f;
     const int64_t blocks_needed = (warps_needed + block / 32 - 1) / (block / 32);
     if (blocks_needed < grid) grid = (int)blocks_needed;
     if (grid < 1) grid = 1;
-    e = cudaMemsetAsync(P.work, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    if (!walk) {
+        e = cudaMemsetAsync(P.work, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+    }
     if (P.out.hit_idx) {
         e = cudaMemsetAsync(P.out.n_hits, 0, sizeof(int64_t), s);
         if (e != cudaSuccess) return e;

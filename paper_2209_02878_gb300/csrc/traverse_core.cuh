@@ -163,6 +163,9 @@ struct TraceCtx {
     int root4;  // root slot for 4-wide traversal
     const float4* nodes;
     const float4* nodes4;  // 4-wide records (see rsi_internal.cuh)
+    const float4* qnodes;  // phased loop: four-way records and their grid
+    const float4* frame;   // (2 entries: origin, scale)
+    bool coarse;           // the grid is too coarse: use `nodes`
     const float4* tris;
     const float4* treelet;
     const float4* snodes;  // shared-memory copy of treelet[0..S)

@@ -4,8 +4,10 @@
 //
 // What bounds it is instruction issue, the divergence between lanes and L1
 // wavefronts (one per 32-byte sector that a lane reads), not DRAM bytes (the
-// tree sits in L1 / L2).  So the loop is split into three phases that each run
-// with many lanes at once:
+// tree sits in L1 / L2).
+//
+// So the loop is split into three phases that each run with many lanes at
+// once:
 //  - node steps: every lane whose current item is a node tests the node's two
 //    child boxes and moves on (leaf children are items like nodes: entered
 //    or pushed, not tested here);
@@ -14,14 +16,29 @@
 //  - refill: finished lanes write their results together and take new
 //    segments that the whole warp has set up 32 at a time in shared memory.
 // A phase runs when kStall lanes cannot take a node step, the one with more
-// lanes waiting first.  Against one loop that does all three for each lane
-// where it stands: 954M -> 610M warp instructions and 14.4 -> 22.9 active
-// lanes on the paper-scale boolean query; boolean 1,177 -> 1,010 us, nearest
-// 2,212 -> 1,615 us there, nearest of the raster 2,291 -> 1,498 us, of the
-// 131,072-triangle terrain with 262,144 segments 238 -> 147 us, of the
-// 1.31M-triangle sphere with 1M segments 1,100 -> 796 us.  NEAREST keeps only
-// the best crossing's position and interval across the loop (its outputs are
-// recomputed once, when written), which takes its spills away.
+// lanes waiting first.  NEAREST keeps only the best crossing's position and
+// interval across the loop (its outputs are recomputed once, when written),
+// which takes its spills away.
+//
+// And a node step takes two levels of the tree at once, from a 64-byte record
+// of the four grandchildren's boxes on a 15-bit grid over the mesh's box: as
+// many bytes and boxes per segment as binary steps on 32-byte grid nodes, but
+// half the steps, each of which costs a ballot, the stack and the loop beside
+// its boxes, and half the chain of dependent reads.  (Exact boxes take twice
+// the bytes.)  The 16-bit half that holds a face becomes a float in [1, 2) by
+// one byte permutation, whose selector also chooses the near or the far face,
+// so the decoding costs what that choice costs anyway.
+//
+// us: one loop for all / phases on exact binary nodes (64 B) / branch-free
+// steps on binary grid nodes (32 B) / on four-way grid nodes (64 B).  The
+// 29,768-triangle terrain with 10M random segments: boolean 1,177 / 1,010 /
+// 823 / 744, count 1,742 / 1,386 / 1,192 / 1,061, nearest 2,212 / 1,615 /
+// 1,426 / 1,336; nearest of its 10M-segment raster 2,291 / 1,498 / 1,387 /
+// 1,345; nearest of the 131,072-triangle terrain and 262,144 segments 238 /
+// 147 / 128 / 114; of the 1.31M-triangle sphere and 1M segments 1,100 / 796 /
+// 684 / 604, its count 1,172 / 965 / 773 / 665.  Boolean: warp instructions
+// 954M / 610M / 564M, L1 wavefronts 240M (65 % of the peak rate) / 253M (79 %) /
+// 148M (51 %), 14.4 / 22.9 / 23.8 active lanes, in the first three.
 #pragma once
 
 #include "traverse_core.cuh"
@@ -29,25 +46,54 @@
 namespace rsi {
 
 constexpr int kDone = (int)0x80000000;  // no item: the segment is finished
-constexpr int kWalkStack = 64;          // a radix tree over 62-bit keys is at most 63 deep
-// Lanes without a node step that end the node phase.  12 / 16 / 20 (72
-// registers): boolean 1,014 / 1,010 / 1,045 us on the 29,768-triangle terrain
-// with 10M random segments, nearest 1,563 / 1,498 / - us under its raster.
-constexpr int kStall = 16;
+// A radix tree over 62-bit keys is at most 63 deep: 32 steps of two levels that
+// push at most three items each, or 63 binary ones that push one.
+constexpr int kWalkStack = 96;
+// Lanes without a node step that end the node phase: fewer keep the lanes
+// busier, more run the other phases fuller (NEAREST has the dearest ones).
+// Boolean and count at 12 / 16 / 20: 758 / 751 / - and 1,072 / 1,056 / - us on
+// the 29,768-triangle terrain with 10M random segments (762 and 1,116 at 20
+// with 72 registers); nearest at 16 / 20 / 24: 1,343 / 1,336 / 1,391 us there,
+// 1,406 / 1,345 / 1,283 of its raster, 610 / 604 / 616 of the sphere.
+template <int MODE>
+constexpr int kStall = MODE == RSI_MODE_NEAREST ? 20 : 16;
+// The same once no segments are left to refill from: 1 / kTail of the lanes
+// still at work.
+constexpr int kTail = 4;
 
-// 72 registers (28 warps per SM): at 64 the loop spills (boolean 1,069 against
-// 1,010 us, count 1,562 against 1,386), at 80 fewer warps hide less (1,034,
-// 1,459); nearest 1,615 us at 72, 1,604 at 64, 1,656 at 80.
-constexpr int kWalkRegs = 72;
+// 80 registers (24 warps per SM): nothing of note spills.  64 / 72 / 80 / 88:
+// boolean 821 / 735 / 744 / 813 us, count 1,211 / 1,080 / 1,061 / 1,155 there;
+// on the 1.31M-triangle sphere with 1M segments boolean 449 / 386 / 360 / 374,
+// count 780 / 700 / 673 / 713, nearest 654 / 661 / 610 / 637.
+constexpr int kWalkRegs = 80;
+
+// Byte selectors that turn the low / high half of a node word into a float.
+constexpr unsigned kSelLo = 0x7104u, kSelHi = 0x7324u, kSelFar = kSelLo ^ kSelHi;
+
+// The nodes' grid (rsi_internal.cuh) has 32,760 steps across the mesh;
+// where more than an eighth of the leaf boxes are below kCoarseSteps steps
+// (fine detail in a far larger mesh) the loop reads the exact binary nodes.
+__device__ __forceinline__ bool walk_coarse(int coarse, int n) { return coarse > n / 8; }
 
 // A lane's segment: end points for the triangle test and, per axis, the
-// constants of the box test
-//   entry parameter = fma(near face, i, n),  exit = fma(far face, i, f).
+// constants of the box test in the grid's coordinates
+//   entry parameter = fma(near face, i, n),  exit = fma(far face, i, f),
+// and the byte selectors that take the near / far face out of a node word.
 struct WalkSeg {
     float ax_, ay_, az_, dx, dy, dz;
     float ix, iy, iz, nx, ny, nz, fx, fy, fz;
+    unsigned swap;        // 32 on odd lanes (walk_node4)
+    unsigned ex, ey, ez;  // selectors of the near faces (far: ^ kSelFar)
     float md;
     bool fp64only;
+    __device__ __forceinline__ void select() {
+        // held as values: recomputed at every node they cost nine instructions
+        ex = ix < 0.f ? kSelHi : kSelLo;
+        ey = iy < 0.f ? kSelHi : kSelLo;
+        ez = iz < 0.f ? kSelHi : kSelLo;
+        swap = (threadIdx.x & 1) * 32u;
+        asm volatile("" : "+r"(ex), "+r"(ey), "+r"(ez));
+    }
     __device__ __forceinline__ float ax() const { return ax_; }
     __device__ __forceinline__ float ay() const { return ay_; }
     __device__ __forceinline__ float az() const { return az_; }
@@ -57,29 +103,36 @@ struct WalkSeg {
     }
 };
 
-// Box-test constants of one axis (u = 2^-24).  With d = fl(b - a) (relative
-// error u) and i = rcp.approx(d) (1 ulp), i = (1 / d_exact)(1 + e), |e| <= 4u.
-// c = fl(a i); a face at x has the exact parameter s = (x - a) / d_exact and
-// x i - c = s (1 + e) + at most u |c|.  The constants are n = -(c + pad) and
-// f = pad - c with pad = 4u |c| + 16u: 4u |c| covers the roundings of c and of
-// n / f, and 16u the relative errors e and the fma's own rounding for every
-// parameter in [0, 1].  So for a box that the exact segment meets at
-// parameters [s0, s1] within [0, 1], the computed entry is below s0 and the
-// computed exit above s1, strictly, and stays so after both are clamped to
-// [0, 1]: `entry < exit` never rejects it.
-//  - |d| < 2^-62 (a zero component, and every tiny one): i = 2^62, pad = 2 +
-//    4u |c|.  A segment inside the slab gets entry <= 0 and exit >= 1; one
-//    that is outside by more than about 2^-61 + 4u |a| is rejected.
-//  - |d| > 2^100 (or infinite) or |c| > 2^100: i = 0, n = -2, f = 2: the
+// Box-test constants of one axis (u = 2^-24) for the segment coordinates
+// X(a) = base + (a - o) s and D = d s, with base = 1 on the grid and o = 0,
+// s = 1, base = 0 (exact) for the exact nodes; d = fl(b - a).
+// i = rcp.approx(D) (1 ulp) is (1 / D_exact)(1 + e), |e| <= 5u (d, D and the
+// reciprocal), and X(a) is off by at most 3u |X(a)| + 2u.  c = fl(X(a) i); a
+// face at X has the exact parameter (X - X_exact(a)) / D_exact, and X i - c is
+// that times (1 + e), up to 4u |c| + 2u |i|.  The constants are n = -(c + pad)
+// and f = pad - c with pad = 8u |c| + 4u |i| + 16u: the first two terms cover
+// those errors and the rounding of n / f (u |c|), and 16u the relative errors
+// e and the fma's own rounding for every parameter in [0, 1].  So for a box
+// that the exact segment meets at parameters [s0, s1] within [0, 1], the
+// computed entry is below s0 and the computed exit above s1, strictly, and
+// stays so after both are clamped to [0, 1]: `entry < exit` never rejects it.
+//  - |D| < 2^-62 (a zero component, and every tiny one): i = 2^62, pad = 2 +
+//    8u |c| + 4u i.  A segment inside the slab gets entry <= 0 and exit >= 1.
+//  - |D| > 2^100 (or infinite) or |c| > 2^100: i = 0, n = -2, f = 2: the
 //    axis never rejects.
-// Empty boxes (both faces +inf) give entry = exit after the clamp (NaN clamps
-// to 0): always rejected.
-__device__ __forceinline__ void walk_axis(float a, float d, float& i, float& n, float& f) {
-    const float ad = fabsf(d);
+// Empty boxes: in the exact nodes both faces are +inf, which is always rejected
+// (entry = exit after the clamp; NaN clamps to 0).  On the grid lo is far beyond
+// hi, and what a segment of a million mesh sizes enters all the same is the
+// null triangle, or triangles without valid vertices: never hit.
+__device__ __forceinline__ void walk_axis(float a, float d, float o, float s, float base, float& i,
+                                          float& n, float& f) {
+    const float X = __fmaf_rn(__fsub_rn(a, o), s, base), D = __fmul_rn(d, s);
+    const float ad = fabsf(D);
     const bool flat = ad < 0x1p-62f;
-    i = flat ? 0x1p62f : rcp_approx(d);
-    const float c = __fmul_rn(a, i);
-    const float pad = __fmaf_rn(fabsf(c), 0x1p-22f, flat ? 2.f : 0x1p-20f);
+    i = flat ? 0x1p62f : rcp_approx(D);
+    const float c = __fmul_rn(X, i);
+    const float pad = __fmaf_rn(fabsf(c), 0x1p-21f,
+                                __fmaf_rn(fabsf(i), 0x1p-22f, flat ? 2.f : 0x1p-20f));
     n = -__fadd_rn(c, pad);
     f = __fsub_rn(pad, c);
     if (!(ad <= 0x1p100f && fabsf(c) <= 0x1p100f)) {
@@ -87,6 +140,20 @@ __device__ __forceinline__ void walk_axis(float a, float d, float& i, float& n, 
         n = -2.f;
         f = 2.f;
     }
+}
+
+// A grid coordinate of a node word as a float: the chosen 16 bits (bit 15 set)
+// become bits 8..23 under 0x3f: 1 + q 2^-15.
+__device__ __forceinline__ float grid_face(unsigned w, unsigned sel) {
+    return __uint_as_float(__byte_perm(w, 0x3f000000u, sel));
+}
+
+// Half a grid record in one 256-bit read-only load.
+__device__ __forceinline__ void ld_qnode(const float4* p, unsigned w[8]) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
+          "=r"(w[7])
+        : "l"(p));
 }
 
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
@@ -105,26 +172,17 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
     return r;
 }
 
-// Entry parameter of the box (clamped to [0, 1]) and whether the segment's
-// part [0, tlim] may meet it.  The clamps come with the fma, so an axis costs
-// two of them and the selection of the near face.
+// Entry parameter of a box with the given near and far faces (clamped to
+// [0, 1]) and whether the segment's part [0, tlim] may meet it.  The clamps
+// come with the fma, so an axis costs two of them and the choice of faces.
 template <bool LIMIT>
-__device__ __forceinline__ bool walk_box(const WalkSeg& s, float lx, float ly, float lz, float hx,
-                                         float hy, float hz, float tlim, float& tn) {
-    const bool gx = s.ix < 0.f, gy = s.iy < 0.f, gz = s.iz < 0.f;
-    tn = max3(fma_sat(gx ? hx : lx, s.ix, s.nx), fma_sat(gy ? hy : ly, s.iy, s.ny),
-              fma_sat(gz ? hz : lz, s.iz, s.nz));
-    float tf = min3(fma_sat(gx ? lx : hx, s.ix, s.fx), fma_sat(gy ? ly : hy, s.iy, s.fy),
-                    fma_sat(gz ? lz : hz, s.iz, s.fz));
+__device__ __forceinline__ bool walk_box(const WalkSeg& s, float ex, float ey, float ez, float gx,
+                                         float gy, float gz, float tlim, float& tn) {
+    tn = max3(fma_sat(ex, s.ix, s.nx), fma_sat(ey, s.iy, s.ny), fma_sat(ez, s.iz, s.nz));
+    float tf = min3(fma_sat(gx, s.ix, s.fx), fma_sat(gy, s.iy, s.fy), fma_sat(gz, s.iz, s.fz));
     if (LIMIT) tf = fminf(tf, tlim);
     return tn < tf;
 }
-
-// Segments set up by a warp and not yet taken by a lane (shared memory, one
-// per warp): four 16-byte words per segment.
-struct WalkStage {
-    float4 q[4][32];
-};
 
 // Leaf items: ~position of a one-triangle leaf, or, with LEAFN (leaf sizes
 // above 1), ~(8 position + count - 1).
@@ -134,10 +192,134 @@ __device__ __forceinline__ int walk_item(int ref, int cnt) {
     return cnt > 0 ? ~((~ref << 3) | (cnt - 1)) : ref;
 }
 
+// A node's children: whether the segment enters each, entry parameters and
+// items.  The two children of the exact binary node:
+template <bool LIMIT, bool LEAFN>
+__device__ __forceinline__ void walk_node2(const TraceCtx& C, const WalkSeg& s, int node, float tlim,
+                                           bool h[2], float t[2], int x[2]) {
+    ulonglong2 q0, q1, q2;
+    int4 rc;
+    ld_node(C.nodes + 4 * (int64_t)node, q0, q1, q2, rc);
+    const float2 lx = up2(q0.x), ly = up2(q0.y), lz = up2(q1.x);
+    const float2 hx = up2(q1.y), hy = up2(q2.x), hz = up2(q2.y);
+    const bool gx = s.ix < 0.f, gy = s.iy < 0.f, gz = s.iz < 0.f;
+    h[0] = walk_box<LIMIT>(s, gx ? hx.x : lx.x, gy ? hy.x : ly.x, gz ? hz.x : lz.x,
+                           gx ? lx.x : hx.x, gy ? ly.x : hy.x, gz ? lz.x : hz.x, tlim, t[0]);
+    h[1] = walk_box<LIMIT>(s, gx ? hx.y : lx.y, gy ? hy.y : ly.y, gz ? hz.y : lz.y,
+                           gx ? lx.y : hx.y, gy ? ly.y : hy.y, gz ? lz.y : hz.y, tlim, t[1]);
+    x[0] = walk_item<LEAFN>(rc.x, rc.z);
+    x[1] = walk_item<LEAFN>(rc.y, rc.w);
+}
+
+// The four children of a 64-byte grid record.  Odd lanes read the halves in
+// the other order (it does not matter which is which): a record's first
+// halves all lie in two of L1's four 32-byte bank groups.
+template <bool LIMIT>
+__device__ __forceinline__ void walk_node4(const TraceCtx& C, const WalkSeg& s, int node, float tlim,
+                                           bool h[4], float t[4], int x[4]) {
+    const float4* p = C.qnodes + 4 * (int64_t)node;
+    unsigned w[16];
+    ld_qnode((const float4*)((uintptr_t)p ^ s.swap), w);
+    ld_qnode((const float4*)((uintptr_t)p ^ s.swap ^ 32u), w + 8);
+    const unsigned gx = s.ex ^ kSelFar, gy = s.ey ^ kSelFar, gz = s.ez ^ kSelFar;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned* c = w + 8 * (k >> 1) + 3 * (k & 1);
+        h[k] = walk_box<LIMIT>(s, grid_face(c[0], s.ex), grid_face(c[1], s.ey),
+                               grid_face(c[2], s.ez), grid_face(c[0], gx), grid_face(c[1], gy),
+                               grid_face(c[2], gz), tlim, t[k]);
+        x[k] = (int)w[8 * (k >> 1) + 6 + (k & 1)];
+    }
+}
+
+// End points and box-test constants of segment i (not md and fp64only);
+// returns whether its coordinates are finite.
+__device__ __forceinline__ bool walk_setup(const TraceCtx& C, int64_t i, WalkSeg& w) {
+    w.ax_ = C.A[3 * i];
+    w.ay_ = C.A[3 * i + 1];
+    w.az_ = C.A[3 * i + 2];
+    const float bx = C.B[3 * i], by = C.B[3 * i + 1], bz = C.B[3 * i + 2];
+    w.dx = __fsub_rn(bx, w.ax_);
+    w.dy = __fsub_rn(by, w.ay_);
+    w.dz = __fsub_rn(bz, w.az_);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 g = make_float4(1.f, 1.f, 1.f, 0.f);
+    if (!C.coarse && C.frame) {
+        o = ld4(C.frame);
+        g = ld4(C.frame + 1);
+    }
+    const float base = C.coarse ? 0.f : 1.f;
+    walk_axis(w.ax_, w.dx, o.x, g.x, base, w.ix, w.nx, w.fx);
+    walk_axis(w.ay_, w.dy, o.y, g.y, base, w.iy, w.ny, w.fy);
+    walk_axis(w.az_, w.dz, o.z, g.z, base, w.iz, w.nz, w.fz);
+    return finite3(w.ax_, w.ay_, w.az_) && finite3(bx, by, bz);
+}
+
+// Segments set up by a warp and not yet taken by a lane (shared memory, one
+// per warp): four 16-byte words per segment.
+struct WalkStage {
+    float4 q[4][32];
+};
+
 // Best crossing of a NEAREST segment: leaf position (kBest64: decided in
 // FP64), and the interval that holds its t.  Everything else about it is
 // recomputed once, when the result is written.
 constexpr unsigned kNoBest = 0xffffffffu, kBest64 = 0x80000000u;
+
+// Test segment i against the triangles of leaf `item`; s.range() is up to
+// date.  Returns true when BOOL found a crossing.
+template <int MODE, bool STATS, bool LEAFN>
+__device__ __forceinline__ bool walk_leaf(const TraceCtx& C, const WalkSeg& s, int64_t i, int item,
+                                          int& count, unsigned& best, float& tlo, float& tlim,
+                                          TravStats& st) {
+    const int pos0 = LEAFN ? (int)((unsigned)~item >> 3) : ~item;
+    const int pos1 = LEAFN ? pos0 + (~item & 7) : pos0;
+    for (int pos = pos0; pos <= pos1; ++pos) {
+        const float4* tp = C.tris + 3 * (int64_t)pos;
+        const float4 a = ld4(tp), b = ld4(tp + 1), c = ld4(tp + 2);
+        float t = 0.f, u = 0.f, v = 0.f, err = 0.f;
+        if (STATS) ++st.tests;
+        int r = mt32(s, a, b, c, MODE == RSI_MODE_NEAREST, t, u, v, err);
+        unsigned code = (unsigned)pos;
+        if (r == 2) {
+            if (STATS) ++st.fp64;
+            const float* pa = C.A + 3 * i;
+            const float* pb = C.B + 3 * i;
+            double tuv[3];
+            r = mt64(pa[0], pa[1], pa[2], pb[0], pb[1], pb[2], a, b, c,
+                     MODE == RSI_MODE_NEAREST ? tuv : nullptr);
+            if (MODE == RSI_MODE_NEAREST && r) {
+                t = (float)tuv[0];
+                err = 0x1p-23f;
+                code |= kBest64;
+            }
+        }
+        if (!r) continue;
+        if (MODE == RSI_MODE_BOOL) {
+            count = 1;
+            return true;
+        }
+        if (MODE == RSI_MODE_COUNT) ++count;
+        if (MODE == RSI_MODE_NEAREST) {
+            bool take = best == kNoBest || t + err < tlo;
+            if (!take && !(t - err > tlim)) {
+                // the intervals overlap: compare the definition's t in FP64,
+                // ties to the lower triangle index
+                const int bpos = (int)(best & ~kBest64);
+                const double tn = exact_t(C.A, C.B, i, C.tris, pos);
+                const double tb = exact_t(C.A, C.B, i, C.tris, bpos);
+                take = tn < tb ||
+                       (tn == tb && f2i(a.w) < f2i(ld4(C.tris + 3 * (int64_t)bpos).w));
+            }
+            if (take) {
+                best = code;
+                tlo = t - err;
+                tlim = fminf(1.f, t + err);
+            }
+        }
+    }
+    return false;
+}
 
 // Outputs of a NEAREST segment with best crossing `best`.
 template <bool STATS>
@@ -151,10 +333,6 @@ __device__ __forceinline__ void walk_nearest_out(const TraceCtx& C, const WalkSe
     if (best != kNoBest) {
         const float4* tp = C.tris + 3 * (int64_t)(best & ~kBest64);
         tri = f2i(ld4(tp).w);
-        Result r;
-        result_init(r);
-        r.best = tri;
-        r.bpos = (int)(best & ~kBest64);
         // the thresholds and their derivation: nearest_values
         const float dd = fmaf(s.dx, s.dx, fmaf(s.dy, s.dy, s.dz * s.dz));
         const float dlen = sqrtf(dd) * 1.0001f;
@@ -209,6 +387,75 @@ __device__ __forceinline__ void walk_nearest_out(const TraceCtx& C, const WalkSe
     if (o.dist) o.dist[i] = dist;
 }
 
+// The stack index is clamped, so that a corrupt tree cannot leave the array;
+// the step bound ends it.
+__device__ __forceinline__ void walk_push(int* stack, int& sp, int x) {
+    sp = min(sp + 1, kWalkStack);
+    stack[sp] = x;
+}
+
+// Node steps of a warp until at most `floor_` lanes have one; returns the
+// lanes that do.  The step has no branches but predicated pushes and a pop: a
+// lane goes on with one of the children that it enters and pushes the others.
+// NEAREST orders them, each pair by entry and the pairs by their first entry
+// (as two binary steps would).
+template <int MODE, bool STATS, bool LEAFN, bool COARSE>
+__device__ __forceinline__ unsigned walk_steps(const TraceCtx& C, const WalkSeg& s, int& cur,
+                                               int& sp, int* stack, float tlim, unsigned& steps,
+                                               unsigned bound, int floor_, TravStats& st) {
+    constexpr bool LIMIT = MODE == RSI_MODE_NEAREST;
+    unsigned inner;
+    do {
+        if (cur >= 0) {
+            if (STATS) ++st.visits;
+            bool h[4];
+            float t[4];
+            int x[4];
+            bool any;
+            if (COARSE) {
+                walk_node2<LIMIT, LEAFN>(C, s, cur, tlim, h, t, x);
+                const bool first0 = h[0] && (!h[1] || t[0] <= t[1]);
+                any = h[0] || h[1];
+                if (h[0] && h[1]) walk_push(stack, sp, first0 ? x[1] : x[0]);
+                cur = first0 ? x[0] : x[1];
+            } else {
+                walk_node4<LIMIT>(C, s, cur, tlim, h, t, x);
+                any = h[0] || h[1] || h[2] || h[3];
+                if (LIMIT) {
+                    const bool a = h[0] && (!h[1] || t[0] <= t[1]);
+                    const bool b = h[2] && (!h[3] || t[2] <= t[3]);
+                    const bool anya = h[0] || h[1], anyb = h[2] || h[3];
+                    const bool two_a = h[0] && h[1], two_b = h[2] && h[3];
+                    const bool f = anya && (!anyb || (a ? t[0] : t[1]) <= (b ? t[2] : t[3]));
+                    const int na = a ? x[0] : x[1], fa = a ? x[1] : x[0];
+                    const int nb = b ? x[2] : x[3], fb = b ? x[3] : x[2];
+                    if (f ? two_b : two_a) walk_push(stack, sp, f ? fb : fa);
+                    if (anya && anyb) walk_push(stack, sp, f ? nb : na);
+                    if (f ? two_a : two_b) walk_push(stack, sp, f ? fa : fb);
+                    cur = f ? na : nb;
+                } else {
+                    cur = x[0];
+                    if (h[1]) {
+                        if (h[0]) walk_push(stack, sp, cur);
+                        cur = x[1];
+                    }
+                    if (h[2]) {
+                        if (h[0] || h[1]) walk_push(stack, sp, cur);
+                        cur = x[2];
+                    }
+                    if (h[3]) {
+                        if (h[0] || h[1] || h[2]) walk_push(stack, sp, cur);
+                        cur = x[3];
+                    }
+                }
+            }
+            if (!any) cur = stack[sp--];
+        }
+        inner = __ballot_sync(0xffffffffu, cur >= 0);
+    } while (__popc(inner) > floor_ && ++steps < bound);
+    return inner;
+}
+
 // Persistent per-warp loop over segments [lo, hi) (work distribution, order,
 // streamed input and compaction as trace_loop).  `start` is the first item
 // of every segment: the Karras root's slot, the whole mesh as one leaf, or
@@ -220,7 +467,8 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    int64_t pool = lo, pool_end = counter ? lo : hi;
+    // segment indices fit 31 bits (walk_fits)
+    unsigned pool = (unsigned)lo, pool_end = counter ? (unsigned)lo : (unsigned)hi;
     bool more = counter != nullptr;  // the counter may hold more chunks
     int head = 0, avail = 0;         // staged segments not yet taken
     unsigned i = kNoBest;            // this lane's segment (kNoBest: none)
@@ -236,12 +484,13 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
     unsigned steps = 0;
     const unsigned bound =
         (unsigned)C.max_visits < 1u << 26 ? 32u * (unsigned)C.max_visits + 64u : 0xffffffffu;
+    unsigned inner = 0u;  // lanes with a node step
     while (true) {
         const unsigned dead = __ballot_sync(FULL, cur == kDone);
-        const unsigned leaf = __ballot_sync(FULL, cur < 0) & ~dead;
+        const unsigned leaf = ~(inner | dead);
         const bool refillable = avail > 0 || pool < pool_end || more;
         const int nd = __popc(dead), nl = __popc(leaf);
-        if (dead == FULL || (refillable && nd >= nl && nd + nl >= kStall)) {
+        if (dead == FULL || (refillable && nd >= nl && nd + nl >= kStall<MODE>)) {
             // ---- refill: results of the finished segments, then new ones
             steps = 0;
             float dist = 0.f, P[3] = {0.f, 0.f, 0.f};
@@ -264,7 +513,7 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
             if (fin) i = kNoBest;
             if (!refillable) break;  // every lane is finished
             unsigned idle = dead;
-            while (idle) {
+            while (true) {
                 if (avail == 0) {  // set up the next segments, one per lane
                     if (pool >= pool_end) {
                         if (!more) break;
@@ -275,24 +524,24 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                             more = false;
                             break;
                         }
-                        pool = (int64_t)b;
-                        pool_end = pool + C.fetch < hi ? pool + C.fetch : hi;
+                        pool = (unsigned)b;
+                        pool_end = (unsigned)min((long long)(b + C.fetch), (long long)hi);
                         // streamed input: see trace_loop
-                        if (C.ready && !wait_flag(C.ready + (pool_end - 1) / C.ready_chunk,
-                                                  C.status, C.wait_polls)) {
+                        if (C.ready &&
+                            !wait_flag(C.ready + (int64_t)(pool_end - 1) / C.ready_chunk, C.status,
+                                       C.wait_polls)) {
                             if (lane == 0) atomicMax(counter, (unsigned long long)hi);
                             pool = pool_end;
                             more = false;
                             break;
                         }
                     }
-                    const int64_t left = pool_end - pool;
-                    const int take = left < 32 ? (int)left : 32;
+                    const int take = (int)min(pool_end - pool, 32u);
                     bool ok = false;
                     WalkSeg w;
                     unsigned k = 0u;
                     if (lane < take) {
-                        int64_t kk = pool + lane;
+                        int64_t kk = (int64_t)pool + lane;
                         bool known = true;
                         if (C.order) {  // a caller's order: entries outside [0, nR) are skipped
                             kk = C.order[kk];
@@ -302,19 +551,7 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                         if (STATS) ++segs;
                         if (known) {
                             k = (unsigned)kk;
-                            w.ax_ = C.A[3 * kk];
-                            w.ay_ = C.A[3 * kk + 1];
-                            w.az_ = C.A[3 * kk + 2];
-                            const float bx = C.B[3 * kk], by = C.B[3 * kk + 1],
-                                        bz = C.B[3 * kk + 2];
-                            ok = finite3(w.ax_, w.ay_, w.az_) && finite3(bx, by, bz) &&
-                                 start != kNoRoot;
-                            w.dx = __fsub_rn(bx, w.ax_);
-                            w.dy = __fsub_rn(by, w.ay_);
-                            w.dz = __fsub_rn(bz, w.az_);
-                            walk_axis(w.ax_, w.dx, w.ix, w.nx, w.fx);
-                            walk_axis(w.ay_, w.dy, w.iy, w.ny, w.fy);
-                            walk_axis(w.az_, w.dz, w.iz, w.nz, w.fz);
+                            ok = walk_setup(C, kk, w) && start != kNoRoot;
                             if (!ok) {  // non-finite segment or empty mesh: a miss
                                 float q0, q1[3];
                                 int tri;
@@ -328,6 +565,7 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                         }
                     }
                     const unsigned good = __ballot_sync(FULL, ok);
+                    __syncwarp();  // the entries before these have been read
                     if (ok) {
                         const int e = __popc(good & lt);
                         sg.q[0][e] = make_float4(w.ax_, w.ay_, w.az_, i2f((int)k));
@@ -341,7 +579,7 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                     avail = __popc(good);
                     if (avail == 0) continue;
                 }
-                const int n = min(avail, __popc(idle));
+                const int want = __popc(idle), n = min(avail, want);
                 const int r = __popc(idle & lt);
                 if (cur == kDone && r < n) {
                     const float4 q0 = sg.q[0][head + r], q1 = sg.q[1][head + r];
@@ -362,6 +600,7 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                     s.nz = q3.y;
                     s.fx = q3.z;
                     s.fy = q3.w;
+                    s.select();
                     cur = start;
                     sp = 0;
                     count = 0;
@@ -370,109 +609,50 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                 }
                 head += n;
                 avail -= n;
+                if (n == want) break;
                 idle = __ballot_sync(FULL, cur == kDone);
-                __syncwarp();  // every lane has read its entry before the next set-up
             }
+            inner = __ballot_sync(FULL, cur >= 0);
             continue;
         }
-        if (nl > 0 && (nd + nl >= kStall || dead + leaf == FULL ||
-                       (!refillable && 4 * nl >= 32 - nd))) {
+        if (nl > 0 && (nd + nl >= kStall<MODE> || inner == 0u || (!refillable && kTail * nl >= 32 - nd))) {
             // ---- triangle tests of the waiting leaves
             if (cur < 0 && cur != kDone) {
                 s.range();
-                const int pos0 = LEAFN ? (int)((unsigned)~cur >> 3) : ~cur;
-                const int pos1 = LEAFN ? pos0 + (~cur & 7) : pos0;
-                bool stop = false;
-                for (int pos = pos0; pos <= pos1; ++pos) {
-                    const float4* tp = C.tris + 3 * (int64_t)pos;
-                    const float4 a = ld4(tp), b = ld4(tp + 1), c = ld4(tp + 2);
-                    float t = 0.f, u = 0.f, v = 0.f, err = 0.f;
-                    if (STATS) ++st.tests;
-                    int r = mt32(s, a, b, c, MODE == RSI_MODE_NEAREST, t, u, v, err);
-                    unsigned code = (unsigned)pos;
-                    if (r == 2) {
-                        if (STATS) ++st.fp64;
-                        const float* pa = C.A + 3 * (int64_t)i;
-                        const float* pb = C.B + 3 * (int64_t)i;
-                        double tuv[3];
-                        r = mt64(pa[0], pa[1], pa[2], pb[0], pb[1], pb[2], a, b, c,
-                                 MODE == RSI_MODE_NEAREST ? tuv : nullptr);
-                        if (MODE == RSI_MODE_NEAREST && r) {
-                            t = (float)tuv[0];
-                            err = 0x1p-23f;
-                            code |= kBest64;
-                        }
-                    }
-                    if (!r) continue;
-                    if (MODE == RSI_MODE_BOOL) {
-                        count = 1;
-                        stop = true;
-                        break;
-                    }
-                    if (MODE == RSI_MODE_COUNT) ++count;
-                    if (MODE == RSI_MODE_NEAREST) {
-                        bool take = best == kNoBest || t + err < tlo;
-                        if (!take && !(t - err > tlim)) {
-                            // the intervals overlap: compare the definition's
-                            // t in FP64, ties to the lower triangle index
-                            const int bpos = (int)(best & ~kBest64);
-                            const double tn = exact_t(C.A, C.B, i, C.tris, pos);
-                            const double tb = exact_t(C.A, C.B, i, C.tris, bpos);
-                            take = tn < tb || (tn == tb && f2i(a.w) <
-                                                   f2i(ld4(C.tris + 3 * (int64_t)bpos).w));
-                        }
-                        if (take) {
-                            best = code;
-                            tlo = t - err;
-                            tlim = fminf(1.f, t + err);
-                        }
-                    }
-                }
-                if (MODE == RSI_MODE_BOOL && stop)
-                    cur = kDone;
-                else
-                    cur = stack[sp--];
+                const bool stop = walk_leaf<MODE, STATS, LEAFN>(C, s, i, cur, count, best, tlo,
+                                                                tlim, st);
+                cur = MODE == RSI_MODE_BOOL && stop ? kDone : stack[sp--];
             }
+            inner = __ballot_sync(FULL, cur >= 0);
             continue;
         }
         // ---- node steps until kStall lanes (a quarter of those left at the
         // end of the work) have none
-        const int alive = refillable ? 32 : 32 - nd;
-        const int floor_ = alive - (refillable ? kStall : max(1, (alive + 3) / 4));
-        do {
-            if (cur >= 0) {
-                ulonglong2 q0, q1, q2;
-                int4 rc;
-                ld_node(C.nodes + 4 * (int64_t)cur, q0, q1, q2, rc);
-                if (STATS) ++st.visits;
-                const float2 lx = up2(q0.x), ly = up2(q0.y), lz = up2(q1.x);
-                const float2 hx = up2(q1.y), hy = up2(q2.x), hz = up2(q2.y);
-                float t0, t1;
-                const bool h0 = walk_box<MODE == RSI_MODE_NEAREST>(s, lx.x, ly.x, lz.x, hx.x, hy.x,
-                                                                   hz.x, tlim, t0);
-                const bool h1 = walk_box<MODE == RSI_MODE_NEAREST>(s, lx.y, ly.y, lz.y, hx.y, hy.y,
-                                                                   hz.y, tlim, t1);
-                const int x0 = walk_item<LEAFN>(rc.x, rc.z), x1 = walk_item<LEAFN>(rc.y, rc.w);
-                if (h0 && h1) {
-                    const bool near0 = t0 <= t1;
-                    cur = near0 ? x0 : x1;
-                    if (sp >= kWalkStack) {  // deeper than any tree: corrupt
-                        atomicCAS(C.status, 0, RSI_ERR_INTERNAL);
-                        cur = kDone;
-                    } else {
-                        stack[++sp] = near0 ? x1 : x0;
-                    }
-                } else if (h0 || h1) {
-                    cur = h0 ? x0 : x1;
-                } else {
-                    cur = stack[sp--];
-                }
-            }
-            if (++steps > bound) {
-                if (lane == 0) atomicCAS(C.status, 0, RSI_ERR_INTERNAL);
-                cur = kDone;
-            }
-        } while (__popc(__ballot_sync(FULL, cur >= 0)) > floor_);
+        const int floor_ = refillable ? 32 - kStall<MODE> : (32 - nd) - max(1, (31 + kTail - nd) / kTail);
+        inner = C.coarse ? walk_steps<MODE, STATS, LEAFN, true>(C, s, cur, sp, stack, tlim, steps,
+                                                                bound, floor_, st)
+                         : walk_steps<MODE, STATS, LEAFN, false>(C, s, cur, sp, stack, tlim, steps,
+                                                                 bound, floor_, st);
+        if (steps >= bound) {
+            if (lane == 0) atomicCAS(C.status, 0, RSI_ERR_INTERNAL);
+            cur = kDone;
+            inner = 0u;
+        }
+    }
+}
+
+// End of a block of a launch whose warps took work from counter[0]: the last
+// block clears it and the count of finished blocks (counter[1]) for the next
+// launch.  A memset before each launch cost as much as a tenth of the
+// smallest queries.  All threads of the block call it.
+__device__ __forceinline__ void walk_finish(unsigned long long* counter) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(counter + 1, 1ull) == (unsigned long long)gridDim.x - 1ull) {
+            counter[0] = 0ull;
+            counter[1] = 0ull;
+        }
     }
 }
 

@@ -24,7 +24,9 @@ def special(seg, rng):
     n = A.shape[0]
     for k, f in enumerate(range(0, n, 7)):
         j = k % 6
-        if j == 0:
+        if k % 13 == 12:  # far longer than any mesh, on every axis
+            A[f], B[f] = (-2e7, -1e7, -3e7), (2e7, 1e7, 3e7)
+        elif j == 0:
             A[f, rng.integers(3)] = (np.nan, np.inf, -np.inf)[k % 3]
         elif j == 1:
             B[f] = A[f]
@@ -80,3 +82,42 @@ def test_terrain_compaction_and_order(n_seg):
         b = bvh.intersect(A, B, mode, launch={"order": order})[key]
         assert torch.equal(a, b), mode
     assert bvh.status() == 0
+
+
+@pytest.mark.parametrize("far", [10.0, 1e5])
+def test_detail_in_a_far_larger_mesh(far):
+    """A fine terrain beside one triangle `far` away: the nodes' grid blurs the
+    terrain's boxes (10: still fine; 1e5: most leaves are below a grid step,
+    and the loop reads the exact nodes)."""
+    mesh, seg, _ = synth.workload_diff(seed=9, n_seg=5000, G=65)
+    n = mesh.V.shape[0]
+    V = np.concatenate([mesh.V, np.float32(far) + np.eye(3, dtype=np.float32)]).astype(np.float32)
+    T = np.concatenate([mesh.T, [[n, n + 1, n + 2]]]).astype(np.int32)
+    A, B = special(seg, np.random.default_rng(1))
+    bvh = rsi.BVH(dev(V), dev(T))
+    compare(bvh, dev(A), dev(B))
+    ref = bvh.intersect(dev(A), dev(B), "nearest", stats=True)["stats"]
+    # no more nodes than the general loop's binary ones, but for the pads
+    gen = bvh.intersect(dev(A), dev(B), "nearest", stats=True, launch={"stack_depth": 32})["stats"]
+    assert ref["node_visits"] <= 1.01 * gen["node_visits"]
+    V[:n, 2] += np.float32(0.01)
+    bvh.refit(dev(V))
+    compare(bvh, dev(A), dev(B))
+    compare(bvh, dev(A), dev(B), compact=True)
+
+
+def test_packets_on_the_same_nodes():
+    for far in (None, 1e5):
+        mesh, seg, _ = synth.workload_diff(seed=10, n_seg=3001, G=33)
+        V, T = mesh.V, mesh.T
+        if far:
+            V = np.concatenate([V, np.float32(far) + np.eye(3)]).astype(np.float32)
+            T = np.concatenate([T, [[len(V) - 3, len(V) - 2, len(V) - 1]]]).astype(np.int32)
+        A, B = (dev(x) for x in special(seg, np.random.default_rng(2)))
+        for leaf in (1, 4):
+            bvh = rsi.BVH(dev(V), dev(T), leaf_size=leaf)
+            for mode, key in (("bool", "flag"), ("count", "count"), ("nearest", "tri")):
+                a = bvh.intersect(A, B, mode, launch={"packet": 1})[key]
+                b = bvh.intersect(A, B, mode, launch={"stack_depth": 32})[key]
+                assert torch.equal(a, b), (far, leaf, mode)
+            assert bvh.status() == 0
