@@ -136,15 +136,21 @@ __global__ void __launch_bounds__(kBuildThreads) k_bounds(MeshArgs ma, TreeBufs 
 #pragma unroll 4
     for (int j = j0 + threadIdx.x; j < j1; j += kBuildThreads) {
         float3 a, bb, c;
-        if (!tri_vertices(md, j, tb.status, a, bb, c)) continue;
+        const bool ok = tri_vertices(md, j, tb.status, a, bb, c);
+        const float3 ce = centroid(a, bb, c);
+        const bool fin = ok && finite3(ce.x, ce.y, ce.z);
+        // k_morton reads it back in order, instead of gathering the vertices
+        // again (26 us at 1.31M triangles); the array is free until the boxes
+        if (!refit)
+            __stcg(tb.pre + (int64_t)md.off + j, make_float4(ce.x, ce.y, ce.z, fin ? 1.f : 0.f));
+        if (!ok) continue;
         v[6] = fminf(v[6], fminf(fminf(a.x, bb.x), c.x));
         v[7] = fminf(v[7], fminf(fminf(a.y, bb.y), c.y));
         v[8] = fminf(v[8], fminf(fminf(a.z, bb.z), c.z));
         v[9] = fmaxf(v[9], fmaxf(fmaxf(a.x, bb.x), c.x));
         v[10] = fmaxf(v[10], fmaxf(fmaxf(a.y, bb.y), c.y));
         v[11] = fmaxf(v[11], fmaxf(fmaxf(a.z, bb.z), c.z));
-        const float3 ce = centroid(a, bb, c);
-        if (!finite3(ce.x, ce.y, ce.z)) continue;
+        if (!fin) continue;
         v[0] = fminf(v[0], ce.x); v[1] = fminf(v[1], ce.y); v[2] = fminf(v[2], ce.z);
         v[3] = fmaxf(v[3], ce.x); v[4] = fmaxf(v[4], ce.y); v[5] = fmaxf(v[5], ce.z);
     }
@@ -226,28 +232,23 @@ __global__ void __launch_bounds__(kBuildThreads) k_morton(MeshArgs ma, TreeBufs 
                 hi = mid - 1;
         }
     }
-    const MeshDesc md = mesh_of(ma, m);
-    const int j = g - md.off;
+    const int axis = ma.M == 1 ? ma.one.height_axis : ma.table[m].height_axis;
     float bnd[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) bnd[k] = tb.bounds[6 * m + k];
-    float3 a, bb, c;
+    const float4 ce = __ldcg(tb.pre + g);  // centroid, w = valid (k_bounds)
     uint32_t code = 0;
-    if (tri_vertices(md, j, tb.status, a, bb, c)) {
-        const float3 ce = centroid(a, bb, c);
-        if (finite3(ce.x, ce.y, ce.z)) {
-            if (md.height_axis == 0) {
-                code = (spread3(quant(ce.x, bnd[0], bnd[3], 1024.f)) << 2) |
-                       (spread3(quant(ce.y, bnd[1], bnd[4], 1024.f)) << 1) |
-                       spread3(quant(ce.z, bnd[2], bnd[5], 1024.f));
-            } else {  // height field: the other two axes, the first one high
-                const bool ax = md.height_axis == 1, az = md.height_axis == 3;
-                const uint32_t q0 = ax ? quant(ce.y, bnd[1], bnd[4], 32768.f)
-                                       : quant(ce.x, bnd[0], bnd[3], 32768.f);
-                const uint32_t q1 = az ? quant(ce.y, bnd[1], bnd[4], 32768.f)
-                                       : quant(ce.z, bnd[2], bnd[5], 32768.f);
-                code = (spread2(q0) << 1) | spread2(q1);
-            }
+    if (ce.w != 0.f) {
+        if (axis == 0) {
+            code = (spread3(quant(ce.x, bnd[0], bnd[3], 1024.f)) << 2) |
+                   (spread3(quant(ce.y, bnd[1], bnd[4], 1024.f)) << 1) |
+                   spread3(quant(ce.z, bnd[2], bnd[5], 1024.f));
+        } else {  // height field: the other two axes, the first one high
+            const uint32_t q0 = axis == 1 ? quant(ce.y, bnd[1], bnd[4], 32768.f)
+                                          : quant(ce.x, bnd[0], bnd[3], 32768.f);
+            const uint32_t q1 = axis == 3 ? quant(ce.y, bnd[1], bnd[4], 32768.f)
+                                          : quant(ce.z, bnd[2], bnd[5], 32768.f);
+            code = (spread2(q0) << 1) | spread2(q1);
         }
     }
     tb.keys[0][g] = ((uint64_t)m << 32) | code;
@@ -310,6 +311,14 @@ __device__ __forceinline__ void store_child_box(float4 lo, float4 hi, float* dst
     dst[3] = hi.x; dst[4] = hi.y; dst[5] = hi.z;
 }
 
+// Two float4 (32-byte aligned) in one 256-bit store: a whole sector, where two
+// 128-bit stores of a warp each send half sectors.
+__device__ __forceinline__ void st2(float4* p, float4 a, float4 b) {
+    asm volatile("st.global.cg.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x),
+                 "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
 __device__ __forceinline__ void write_node(float4* nodes, int slot, float4 l0, float4 h0,
                                            int ref0, int cnt0, float4 l1, float4 h1, int ref1,
                                            int cnt1) {
@@ -322,34 +331,32 @@ __device__ __forceinline__ void write_node(float4* nodes, int slot, float4 l0, f
     f[15] = i2f(cnt1);
     // the two children's coordinates interleaved in pairs (see rsi_internal.cuh)
     float4* o = nodes + 4 * (int64_t)slot;
-    __stcg(o + 0, make_float4(f[0], f[6], f[1], f[7]));
-    __stcg(o + 1, make_float4(f[2], f[8], f[3], f[9]));
-    __stcg(o + 2, make_float4(f[4], f[10], f[5], f[11]));
-    __stcg(o + 3, make_float4(f[12], f[13], f[14], f[15]));
+    st2(o, make_float4(f[0], f[6], f[1], f[7]), make_float4(f[2], f[8], f[3], f[9]));
+    st2(o + 2, make_float4(f[4], f[10], f[5], f[11]), make_float4(f[12], f[13], f[14], f[15]));
 }
 
 // One axis of a child box on the grid, rounded outward: lo | hi << 16, each with
 // bit 15 set.  (x - o) s carries two roundings, below 2^-8 of a step, so the
 // 1/16 step leaves the grid box around the exact one; an empty box becomes
 // lo = 32767, hi = 0, which no segment enters.
-__device__ __forceinline__ uint32_t grid_axis(float lo, float hi, float o, float s) {
-    if (lo > hi) return 0x8000ffffu;
+__device__ __forceinline__ int grid_axis(float lo, float hi, float o, float s) {
+    if (lo > hi) return (int)0x8000ffffu;
     const float a = __fmul_rn(__fmul_rn(__fsub_rn(lo, o), s), 32768.f);
     const float b = __fmul_rn(__fmul_rn(__fsub_rn(hi, o), s), 32768.f);
     const uint32_t q0 = (uint32_t)fminf(fmaxf(floorf(a - 0.0625f), 0.f), 32767.f);
     const uint32_t q1 = (uint32_t)fmaxf(fminf(ceilf(b + 0.0625f), 32767.f), 0.f);
-    return (0x8000u | q0) | (0x8000u | q1) << 16;
+    return (int)((0x8000u | q0) | (0x8000u | q1) << 16);
 }
 
 // Half `h` of qnodes: boxes and items of two siblings.
 __device__ __forceinline__ void write_half(const TreeBufs& tb, int m, int h, float4 l0, float4 h0,
                                            int x0, float4 l1, float4 h1, int x1) {
     const float4 o = tb.frame[2 * m], s = tb.frame[2 * m + 1];
-    uint4* q = (uint4*)(tb.qnodes + 2 * (int64_t)h);
-    __stcg(q, make_uint4(grid_axis(l0.x, h0.x, o.x, s.x), grid_axis(l0.y, h0.y, o.y, s.y),
-                         grid_axis(l0.z, h0.z, o.z, s.z), grid_axis(l1.x, h1.x, o.x, s.x)));
-    __stcg(q + 1, make_uint4(grid_axis(l1.y, h1.y, o.y, s.y), grid_axis(l1.z, h1.z, o.z, s.z),
-                             (uint32_t)x0, (uint32_t)x1));
+    st2(tb.qnodes + 2 * (int64_t)h,
+        make_float4(i2f(grid_axis(l0.x, h0.x, o.x, s.x)), i2f(grid_axis(l0.y, h0.y, o.y, s.y)),
+                    i2f(grid_axis(l0.z, h0.z, o.z, s.z)), i2f(grid_axis(l1.x, h1.x, o.x, s.x))),
+        make_float4(i2f(grid_axis(l1.y, h1.y, o.y, s.y)), i2f(grid_axis(l1.z, h1.z, o.z, s.z)),
+                    i2f(x0), i2f(x1)));
 }
 
 __device__ __forceinline__ int leaf_item(const TreeBufs& tb, int pos, int cnt) {
@@ -455,8 +462,7 @@ __device__ __forceinline__ void finish_node(const TreeBufs& tb, const MeshDesc& 
     const int ref1 = z1 <= L ? f1 : cc.y, cnt1 = z1 <= L ? z1 : 0;
     float ul[3] = {l0[0], l0[1], l0[2]}, uh[3] = {h0[0], h0[1], h0[2]};
     merge_box(ul, uh, f4(l1), f4(h1));
-    __stcg(tb.nbox + 2 * (int64_t)node, f4(ul));
-    __stcg(tb.nbox + 2 * (int64_t)node + 1, f4(uh));
+    st2(tb.nbox + 2 * (int64_t)node, f4(ul), f4(uh));
     write_node(tb.nodes, node, f4(l0), f4(h0), ref0, cnt0, f4(l1), f4(h1), ref1, cnt1);
     if (z0 + z1 > L)  // else collapsed into a leaf
         write_qnode(tb, m, node, node == md.off, f4(l0), f4(h0), ref0, cnt0, f4(l1), f4(h1), ref1,
@@ -469,25 +475,37 @@ __device__ __forceinline__ void finish_node(const TreeBufs& tb, const MeshDesc& 
     }
 }
 
-// Shared-memory sparse table of one block's leaf boxes: level k holds the
-// union of the 2^k boxes starting at each position (kBoxBlock - 2^k + 1
-// entries), levels packed one after another, six float planes (lo xyz,
-// hi xyz).  The union over any range [a, b] of the block is that of two
-// overlapping entries of level floor(log2(b - a + 1)).
-constexpr int kBoxLevels = 10;  // log2(kBoxBlock) + 1
-static_assert(1 << (kBoxLevels - 1) == kBoxBlock, "kBoxBlock is a power of two");
-__host__ __device__ constexpr int st_level(int k) { return k * (kBoxBlock + 1) - ((1 << k) - 1); }
+// Shared-memory table of one block's leaf boxes: level k holds the union of the
+// 4^k boxes starting at each position (kBoxBlock - 4^k + 1 entries), levels
+// packed one after another, six float planes (lo xyz, hi xyz).  The union over
+// any range of the block is that of at most four overlapping entries of the
+// largest level that fits it.  (With windows of 2^k the table takes 10 levels
+// and 110 KB, two entries a query and twice the barriers; two blocks fit an SM
+// instead of four.  What bounds the pass is the gather of the triangles and its 350 B of
+// stores per triangle: 131 us at 1.31M triangles with those levels and 128-bit
+// stores, 139 with these and the four-way records added, 113 with whole-sector
+// stores, st2.)
+constexpr int kBoxLevels = 5;  // windows 1, 4, 16, 64, 256
+__host__ __device__ constexpr int st_level(int k) {
+    return k * (kBoxBlock + 1) - ((1 << (2 * k)) - 1) / 3;
+}
+static_assert(1 << (2 * (kBoxLevels - 1)) <= kBoxBlock && kBoxBlock < 1 << (2 * kBoxLevels),
+              "the levels cover a block");
 constexpr int kStEntries = st_level(kBoxLevels);
 constexpr size_t kBoxSmem = sizeof(float) * 6 * kStEntries + 2 * sizeof(int2) * kBoxBlock;
 
 // Union of the leaf boxes at block positions [a, b] (a <= b).
 __device__ __forceinline__ void st_query(const float* st, int a, int b, float l[3], float h[3]) {
-    const int k = 31 - __clz(b - a + 1);
-    const int i = st_level(k) + a, j = st_level(k) + b - (1 << k) + 1;
+    const int k = (31 - __clz(b - a + 1)) >> 1, w = 1 << (2 * k);
+    const float* p = st + st_level(k);
+    const int i0 = a, i3 = b - w + 1;  // first and last window
+    const int i1 = min(a + w, i3), i2 = min(a + 2 * w, i3);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        l[c] = fminf(st[c * kStEntries + i], st[c * kStEntries + j]);
-        h[c] = fmaxf(st[(3 + c) * kStEntries + i], st[(3 + c) * kStEntries + j]);
+        const float* q = p + c * kStEntries;
+        l[c] = fminf(fminf(q[i0], q[i1]), fminf(q[i2], q[i3]));
+        q += 3 * kStEntries;
+        h[c] = fmaxf(fmaxf(q[i0], q[i1]), fmaxf(q[i2], q[i3]));
     }
 }
 
@@ -539,8 +557,7 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
             hi[1] = fmaxf(fmaxf(a.y, b.y), c.y);
             hi[2] = fmaxf(fmaxf(a.z, b.z), c.z);
         }
-        __stcg(tb.lbox + 2 * (int64_t)g, f4(lo));
-        __stcg(tb.lbox + 2 * (int64_t)g + 1, f4(hi));
+        st2(tb.lbox + 2 * (int64_t)g, f4(lo), f4(hi));
         if (ok) {
             const float4 s = tb.frame[2 * m + 1];
             const float e = fmaxf(fmaxf((hi[0] - lo[0]) * s.x, (hi[1] - lo[1]) * s.y),
@@ -582,16 +599,18 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
             }
         }
     }
+#pragma unroll
     for (int k = 1; k < kBoxLevels; ++k) {
         __syncthreads();
-        const int h = 1 << (k - 1);
-        if (tid <= kBoxBlock - 2 * h) {
+        const int w = 1 << (2 * (k - 1));
+        if (tid <= kBoxBlock - 4 * w) {
             const int s = st_level(k - 1) + tid, d = st_level(k) + tid;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                st[c * kStEntries + d] = fminf(st[c * kStEntries + s], st[c * kStEntries + s + h]);
-                st[(3 + c) * kStEntries + d] =
-                    fmaxf(st[(3 + c) * kStEntries + s], st[(3 + c) * kStEntries + s + h]);
+                const float* q = st + c * kStEntries + s;
+                st[c * kStEntries + d] = fminf(fminf(q[0], q[w]), fminf(q[2 * w], q[3 * w]));
+                q += 3 * kStEntries;
+                st[(3 + c) * kStEntries + d] = fmaxf(fmaxf(q[0], q[w]), fmaxf(q[2 * w], q[3 * w]));
             }
         }
     }
@@ -599,11 +618,9 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
     if (g >= N) return;
     float l0[3], h0[3];
     st_query(st, 0, tid, l0, h0);
-    __stcg(tb.pre + 2 * (int64_t)g, f4(l0));
-    __stcg(tb.pre + 2 * (int64_t)g + 1, f4(h0));
+    st2(tb.pre + 2 * (int64_t)g, f4(l0), f4(h0));
     st_query(st, tid, kBoxBlock - 1, l0, h0);
-    __stcg(tb.suf + 2 * (int64_t)g, f4(l0));
-    __stcg(tb.suf + 2 * (int64_t)g + 1, f4(h0));
+    st2(tb.suf + 2 * (int64_t)g, f4(l0), f4(h0));
     if (!local) return;
     // the record of slot g: children [first, gam] and [gam + 1, last]
     const int2 rg = srg[tid], cc = sch[tid];

@@ -59,8 +59,8 @@ namespace rsi {
 constexpr int kMaxLeaf = 8;
 constexpr int kTreeletMax = 2048;   // nodes in the breadth-first top treelet
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys per tile
+constexpr int kSortItems = 8;
+constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
 constexpr int kSortTileMin = kSortThreads * 4;         // 1024 keys per tile (small sorts)
 constexpr int kSortBins = 256;
 constexpr int kBuildThreads = 256;

@@ -11,6 +11,13 @@
 //                  scatter to base + tile offset + rank.
 // With at most kSortFuseTiles tiles the scan kernel is skipped: every
 // scatter block sums the (few) tile histograms of its digit itself.
+//
+// What bounds the scatter is its stores: 35 us a pass at 1.31M 12-byte entries
+// when each lane stores to its own sector, 22 when the tile is ordered by digit
+// in shared memory first (and 16 either way where the digits are already
+// nearly in order).  The build of that mesh as a graph: 434 -> 359 us with the
+// box pass's whole-sector stores and the kept centroids (build.cu); the order
+// of 1,000,003 segments 100 -> 74 us, of 262,144 96 -> 43 us, of 65,536 62 -> 35.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -20,7 +27,8 @@
 
 namespace rsi {
 
-template <typename K, int ITEMS>
+// FUSED: hist[tile][d], so that the scatter's sums over the tiles read rows.
+template <typename K, int ITEMS, bool FUSED>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const K* __restrict__ keys, int n,
                                                             int shift, uint32_t* __restrict__ hist,
                                                             int ntiles) {
@@ -28,13 +36,18 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const K* __restrict_
     h[threadIdx.x] = 0;
     __syncthreads();
     const int base = blockIdx.x * kSortThreads * ITEMS;
-#pragma unroll 4
+    uint32_t dig[ITEMS];
+#pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
         const int pos = base + it * kSortThreads + threadIdx.x;
-        if (pos < n) atomicAdd(&h[(uint32_t)(keys[pos] >> shift) & 0xffu], 1u);
+        dig[it] = pos < n ? (uint32_t)(keys[pos] >> shift) & 0xffu : kSortBins;
     }
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it)
+        if (dig[it] < kSortBins) atomicAdd(&h[dig[it]], 1u);
     __syncthreads();
-    hist[threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    hist[FUSED ? blockIdx.x * kSortBins + threadIdx.x : threadIdx.x * ntiles + blockIdx.x] =
+        h[threadIdx.x];
 }
 
 // Block-wide exclusive scan of one value per thread (blockDim.x <= 1024).
@@ -84,7 +97,7 @@ static __global__ void __launch_bounds__(256) k_sort_scan(uint32_t* __restrict__
     if (threadIdx.x == 0) totals[blockIdx.x] = tot;
 }
 
-constexpr int kSortFuseTiles = 64;
+constexpr int kSortFuseTiles = 16;  // build of 29,768 triangles (30 tiles) 64 us fused, 60 not
 
 template <typename K, int ITEMS, bool FUSED>
 __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
@@ -92,17 +105,24 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
     uint32_t* __restrict__ vout, int n, int shift, const uint32_t* __restrict__ hist,
     const uint32_t* __restrict__ totals, int ntiles) {
     constexpr int W = kSortThreads / 32;
+    // Large sorts order the tile by digit in shared memory first, so that a
+    // warp's stores run along a few output runs instead of touching a sector
+    // per lane.
+    constexpr bool REORDER = ITEMS > 4;
     __shared__ uint32_t cnt[W][kSortBins];
+    __shared__ K sk[REORDER ? kSortThreads * ITEMS : 1];
+    __shared__ uint32_t sv[REORDER ? kSortThreads * ITEMS : 1];
+    __shared__ uint32_t gbase[REORDER ? kSortBins : 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int q = threadIdx.x; q < W * kSortBins; q += kSortThreads) (&cnt[0][0])[q] = 0;
     // this tile's offset within digit d (FUSED: summed here from the raw tile
     // histograms) and the digit total; kSortThreads == bins, thread = digit
     uint32_t toff, dtot;
     if (FUSED) {
-        const uint32_t* row = hist + (size_t)threadIdx.x * ntiles;
         toff = dtot = 0u;
+#pragma unroll 8
         for (int q = 0; q < ntiles; ++q) {
-            const uint32_t x = row[q];
+            const uint32_t x = hist[q * kSortBins + threadIdx.x];
             toff += q < (int)blockIdx.x ? x : 0u;
             dtot += x;
         }
@@ -115,11 +135,18 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
     const int wbase = blockIdx.x * (kSortThreads * ITEMS) + w * (32 * ITEMS);
     const uint32_t lt = (1u << lane) - 1u;
     uint32_t local[ITEMS];
+    K key[ITEMS];
+    uint32_t val[ITEMS];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
         const int pos = wbase + it * 32 + lane;
-        const bool valid = pos < n;
-        const uint32_t d = valid ? ((uint32_t)(kin[pos] >> shift) & 0xffu) : 0x100u;
+        key[it] = pos < n ? kin[pos] : (K)0;
+        val[it] = pos < n ? vin[pos] : 0u;
+    }
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const bool valid = wbase + it * 32 + lane < n;
+        const uint32_t d = valid ? ((uint32_t)(key[it] >> shift) & 0xffu) : 0x100u;
         const uint32_t peers = __match_any_sync(0xffffffffu, d);
         const uint32_t rank = __popc(peers & lt);
         const uint32_t c = valid ? cnt[w][d] : 0u;
@@ -129,26 +156,56 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
         local[it] = c + rank;
     }
     __syncthreads();
-    {
-        const int d = threadIdx.x;
-        uint32_t run = dbase + toff;
+    // this tile's keys of digit d, by warp, and (REORDER) where digit d starts
+    // in the tile
+    const int d0 = threadIdx.x;
+    uint32_t mine = 0;
 #pragma unroll
-        for (int q = 0; q < W; ++q) {
-            const uint32_t x = cnt[q][d];
-            cnt[q][d] = run;
-            run += x;
+    for (int q = 0; q < W; ++q) mine += cnt[q][d0];
+    uint32_t run = dbase + toff;
+    if (REORDER) {
+        const uint32_t start = block_scan_u32(mine, nullptr);
+        gbase[d0] = run - start;  // global position of digit d0's run less its local one
+        run = start;
+    }
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+        const uint32_t x = cnt[q][d0];
+        cnt[q][d0] = run;
+        run += x;
+    }
+    __syncthreads();
+    if (!REORDER) {
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            if (wbase + it * 32 + lane < n) {
+                const uint32_t d = (uint32_t)(key[it] >> shift) & 0xffu;
+                const uint32_t o = cnt[w][d] + local[it];
+                kout[o] = key[it];
+                vout[o] = val[it];
+            }
+        }
+        return;
+    }
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        if (wbase + it * 32 + lane < n) {
+            const uint32_t d = (uint32_t)(key[it] >> shift) & 0xffu;
+            const uint32_t o = cnt[w][d] + local[it];
+            sk[o] = key[it];
+            sv[o] = val[it];
         }
     }
     __syncthreads();
+    const int have = min(n - (int)blockIdx.x * (kSortThreads * ITEMS), kSortThreads * ITEMS);
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int pos = wbase + it * 32 + lane;
-        if (pos < n) {
-            const K k = kin[pos];
-            const uint32_t d = (uint32_t)(k >> shift) & 0xffu;
-            const uint32_t o = cnt[w][d] + local[it];
+        const int p = it * kSortThreads + threadIdx.x;
+        if (p < have) {
+            const K k = sk[p];
+            const uint32_t o = gbase[(uint32_t)(k >> shift) & 0xffu] + (uint32_t)p;
             kout[o] = k;
-            vout[o] = vin[pos];
+            vout[o] = sv[p];
         }
     }
 }
@@ -156,7 +213,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
 // Sort keys[0] / vals[0] (n entries) over the digits at `shifts`; buffers
 // keys[1] / vals[1] are ping-pong space; *out receives the index of the
 // buffer pair holding the result.  Tiles hold 1024 keys below 2^18 keys (more
-// blocks for small sorts), 4096 above.  hist: kSortBins * ceil(n / 1024)
+// blocks for small sorts: from 2^17 on, the build of 131,072 triangles takes 83
+// us instead of 78), 2048 above (4096: 362 against 359 us at 1.31M).  hist: kSortBins * ceil(n / 1024)
 // words, totals: kSortBins words.
 template <typename K, int ITEMS>
 static cudaError_t radix_sort_tiles(K* keys[2], uint32_t* vals[2], int n, const int* shifts,
@@ -166,13 +224,15 @@ static cudaError_t radix_sort_tiles(K* keys[2], uint32_t* vals[2], int n, const 
     const int ntiles = (n + tile - 1) / tile;
     int cur = 0;
     for (int p = 0; p < np && n > 0; ++p) {
-        k_sort_hist<K, ITEMS><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p], hist,
-                                                              ntiles);
         if (ntiles <= kSortFuseTiles) {
+            k_sort_hist<K, ITEMS, true><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p],
+                                                                        hist, ntiles);
             k_sort_scatter<K, ITEMS, true><<<ntiles, kSortThreads, 0, s>>>(
                 keys[cur], vals[cur], keys[1 - cur], vals[1 - cur], n, shifts[p], hist, totals,
                 ntiles);
         } else {
+            k_sort_hist<K, ITEMS, false><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p],
+                                                                         hist, ntiles);
             k_sort_scan<<<kSortBins, 256, 0, s>>>(hist, ntiles, totals);
             k_sort_scatter<K, ITEMS, false><<<ntiles, kSortThreads, 0, s>>>(
                 keys[cur], vals[cur], keys[1 - cur], vals[1 - cur], n, shifts[p], hist, totals,
