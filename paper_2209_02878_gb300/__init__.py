@@ -11,6 +11,7 @@ crossing with triangle id, (t, u, v), point and distance (``barycentric``).
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes as C
 
 import numpy as np
@@ -93,15 +94,28 @@ def use_torch_allocator(enable: bool = True):
 
 
 def _vp(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+_HERE = contextlib.nullcontext()
+
+
+def _on(device):
+    """Context in which `device` is the current one; nothing to do when it
+    already is (torch.cuda.device takes longer than a launch)."""
+    return _HERE if device.index == torch.cuda.current_device() else torch.cuda.device(device)
 
 
 def _check_tensor(t, name, dtype, cols=3):
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous()
+            and (not cols or (t.dim() == 2 and t.shape[1] == cols))):
+        return t
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if not t.is_cuda:
@@ -124,23 +138,27 @@ def _mode(mode) -> int:
         raise ValueError(f"unknown mode {mode!r}; use one of {sorted(MODES)}") from None
 
 
+_NO_OPTIONS = _abi.rsi_launch_opts()  # all defaults; only ever read
+
+
 def _launch(launch, n=None, device=None):
     """rsi_launch_opts from a dict; "order" is an int32 CUDA tensor of n
     entries (a processing order, e.g. from BVH.segment_order)."""
+    if not launch:
+        return _NO_OPTIONS
     lo = _abi.rsi_launch_opts()
-    if launch:
-        for k, v in launch.items():
-            if k == "order":
-                if v is None:
-                    continue
-                _check_tensor(v, "order", torch.int32, cols=0)
-                if v.dim() != 1 or (n is not None and v.shape[0] != n):
-                    raise ValueError("order must be a 1-D int32 tensor with one entry per segment")
-                if device is not None and v.device != device:
-                    raise ValueError("order must be on the segments' device")
-                lo.order = v.data_ptr()
-            else:
-                setattr(lo, k, int(v))
+    for k, v in launch.items():
+        if k == "order":
+            if v is None:
+                continue
+            _check_tensor(v, "order", torch.int32, cols=0)
+            if v.dim() != 1 or (n is not None and v.shape[0] != n):
+                raise ValueError("order must be a 1-D int32 tensor with one entry per segment")
+            if device is not None and v.device != device:
+                raise ValueError("order must be on the segments' device")
+            lo.order = v.data_ptr()
+        else:
+            setattr(lo, k, int(v))
     return lo
 
 
@@ -169,12 +187,15 @@ def _alloc_outputs(mode: int, n: int, dev, compact: bool, hit_cap):
     return o
 
 
+_OUT_POINTERS = frozenset(("flag", "count", "tri", "tuv", "point", "dist", "hit_idx", "n_hits",
+                           "hit_tri", "hit_dist", "hit_point", "hit_count"))
+
+
 def _rsi_output(o) -> _abi.rsi_output:
     r = _abi.rsi_output()
-    for k in ("flag", "count", "tri", "tuv", "point", "dist", "hit_idx", "n_hits", "hit_tri",
-              "hit_dist", "hit_point", "hit_count"):
-        if k in o and o[k] is not None:
-            setattr(r, k, o[k].data_ptr())
+    for k, v in o.items():
+        if k in _OUT_POINTERS and v is not None:
+            setattr(r, k, v.data_ptr())
     r.hit_cap = int(o.get("hit_cap", 0))
     return r
 
@@ -197,7 +218,7 @@ class BVH:
         self.leaf_size, self.top_levels, self.height_axis = leaf_size, top_levels, height_axis
         opts = _abi.rsi_build_opts(int(leaf_size), int(top_levels), int(height_axis))
         h = C.c_void_p()
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_bvh_create(self.nV, self.nT, C.byref(opts), _stream(stream),
                                                 C.byref(h)), "rsi_bvh_create")
         self._h = h
@@ -220,7 +241,7 @@ class BVH:
         _check_tensor(T, "T", torch.int32)
         if V.shape[0] != self.nV or T.shape[0] != self.nT:
             raise ValueError("build: sizes differ from the handle's")
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_bvh_build(self._h, _vp(V), _vp(T), _stream(stream)),
                        "rsi_bvh_build")
         self.T = T
@@ -233,7 +254,7 @@ class BVH:
         _check_tensor(V, "V", torch.float32)
         if V.shape[0] != self.nV:
             raise ValueError("refit: vertex count differs from the handle's")
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_refit(self._h, _vp(V), _vp(self.T), _stream(stream)),
                        "rsi_refit")
         self._vkey = self._key(V)
@@ -254,7 +275,7 @@ class BVH:
 
     def status(self, stream=None) -> int:
         """Synchronise and return (then clear) the device-side status word."""
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             return int(self._lib.rsi_bvh_status(self._h, _stream(stream)))
 
     def info(self) -> dict:
@@ -276,7 +297,7 @@ class BVH:
         o = out if out is not None else _alloc_outputs(m, n, A.device, compact, hit_cap)
         ro = _rsi_output(o)
         lo = _launch(launch, n, A.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             if stats:
                 st = _abi.rsi_stats()
                 _abi.check(self._lib.rsi_intersect_stats(self._h, _vp(A), _vp(B), n, m,
@@ -301,7 +322,7 @@ class BVH:
             raise ValueError("A and B must have the same shape")
         n = int(A.shape[0])
         order = torch.empty(n, dtype=torch.int32, device=A.device)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_segment_order(self._h, _vp(A), _vp(B), n, int(bits),
                                                    _vp(order), _stream(stream)),
                        "rsi_segment_order")
@@ -338,7 +359,7 @@ class BVH:
                        "dist": torch.empty(n, dtype=torch.float32, pin_memory=pin)}
         ro = _rsi_output(out)
         lo = _launch(launch)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_intersect_host(self._h, _vp(A), _vp(B), n, m, C.byref(ro),
                                                     int(chunk), C.byref(lo), _stream(stream)),
                        "rsi_intersect_host")
@@ -350,7 +371,7 @@ class BVH:
         _check_tensor(P, "P", torch.float32)
         out = torch.empty(int(P.shape[0]), dtype=torch.uint8, device=P.device)
         lo = _launch(launch)
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_points_inside(self._h, _vp(P), int(P.shape[0]), _vp(out),
                                                    C.byref(lo), _stream(stream)),
                        "rsi_points_inside")
@@ -366,7 +387,7 @@ class BVH:
                  nbox=np.zeros((max(n - 1, 0), 6), np.float32),
                  lbox=np.zeros((n, 6), np.float32), nodes=np.zeros((max(n, 1), 16), np.float32))
         p = {k: v.ctypes.data_as(C.c_void_p) for k, v in o.items()}
-        with torch.cuda.device(self.device):
+        with _on(self.device):
             _abi.check(self._lib.rsi_bvh_export(self._h, _stream(stream), p["bounds"], p["codes"],
                                                 p["order"], p["left"], p["right"], p["range"],
                                                 p["nbox"], p["lbox"], p["nodes"]),
@@ -417,7 +438,7 @@ def intersect_backward(V, T, A, B, tri, grad_point=None, grad_tuv=None, grad_V=N
     gV = grad_V if grad_V is not None else torch.zeros_like(V)
     gA = torch.empty_like(A)
     gB = torch.empty_like(B)
-    with torch.cuda.device(V.device):
+    with _on(V.device):
         _abi.check(lib.rsi_intersect_backward(_vp(V), int(V.shape[0]), _vp(T), int(T.shape[0]),
                                               _vp(A), _vp(B), n, _vp(tri), _vp(grad_point),
                                               _vp(grad_tuv), _vp(gV), _vp(gA), _vp(gB),
@@ -438,13 +459,13 @@ class RSIFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, V, A, B, T, bvh, order=None):
+        V, A, B = V.detach(), A.detach(), B.detach()
         if bvh is None:
-            bvh = BVH(V.detach(), T)
+            bvh = BVH(V, T)
         else:
-            bvh.sync(V.detach(), T)
-        o = bvh.intersect(A.detach(), B.detach(), "nearest",
-                          launch={"order": order} if order is not None else None)
-        ctx.save_for_backward(V.detach(), A.detach(), B.detach(), T, o["tri"])
+            bvh.sync(V, T)
+        o = bvh.intersect(A, B, "nearest", launch={"order": order} if order is not None else None)
+        ctx.save_for_backward(V, A, B, T, o["tri"])
         ctx.mark_non_differentiable(o["tri"])
         return o["point"], o["tuv"], o["tri"]
 
