@@ -1016,7 +1016,9 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
     });
     std::vector<rsi::BatchItemDev> dev(n);
     std::vector<rsi::BatchTile> tiles;
-    bool walk = true;
+    bool walk = cfg.stack == 64;  // the phased loop takes every item
+    for (int k = 0; k < n; ++k) walk = walk && rsi::walk_fits(items[k].nR, N, leaf);
+    const int64_t tile = walk ? rsi::kBatchTile : rsi::kBatchTileGeneral;
     int64_t mode_first[3] = {0, 0, 0}, mode_tiles[3] = {0, 0, 0};
     for (int q = 0; q < n; ++q) {
         const int k = ord[q];
@@ -1028,16 +1030,15 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n, const rsi_bu
         d.root = it.nT > 0 ? (int)(table[k].off + it.nT - 1) : rsi::kNoRoot;
         d.n = (int)it.nT;
         d.start = rsi::walk_start(table[k].off, (int)it.nT, leaf);
-        walk = walk && rsi::walk_fits(it.nR, N, leaf);
         d.mode = it.mode;
         d.out = trav_out((rsi_mode)it.mode, &it.out);
-        for (int64_t lo = 0; lo < it.nR; lo += rsi::kBatchTile) {
+        for (int64_t lo = 0; lo < it.nR; lo += tile) {
             if (mode_tiles[it.mode]++ == 0) mode_first[it.mode] = (int64_t)tiles.size();
             rsi::BatchTile t;
             t.item = k;
             t.pad = 0;
             t.lo = lo;
-            t.hi = lo + rsi::kBatchTile < it.nR ? lo + rsi::kBatchTile : it.nR;
+            t.hi = lo + tile < it.nR ? lo + tile : it.nR;
             tiles.push_back(t);
         }
     }

@@ -1,5 +1,5 @@
 // Batched traversal: many independent (mesh, segments, mode) problems in one
-// persistent launch.  The work is a list of tiles (up to kBatchTile segments
+// persistent launch per mode.  The work is a list of tiles (a few hundred segments
 // of one item) ordered by decreasing estimated cost per segment (log2 N_t,
 // NEAREST and COUNT weighted above BOOL) so the expensive tiles start first;
 // each warp pulls the next tile from one atomic counter and runs the same
@@ -70,31 +70,36 @@ __global__ void __maxnreg__(128) k_batch(BatchParams P) {
 // that mode's tiles, so that each keeps its own register count.  Inlined into
 // one kernel the three need 128 registers: 1,790 us on 16 meshes with 3.5M
 // segments, and 2,178 us out of line (the calls save too much); the general
-// loop, inlined at 128, 2,265 us.
+// loop, inlined at 128, 2,265 us; side by side at 80 registers with tiles of
+// 1,024, each run dry, 1,549; as below 1,143.
+//
+// A warp goes on with the tiles of one item (they are consecutive in the list)
+// without letting its lanes run dry in between; a tile of another item waits
+// until they have finished.
 template <int MODE, bool LEAFN>
-__global__ void __maxnreg__(kWalkRegs) k_batch_walk(BatchParams P) {
+__global__ void __maxnreg__(kBatchRegs) k_batch_walk(BatchParams P) {
     extern __shared__ float4 stage4[];
     WalkStage& sg = ((WalkStage*)stage4)[threadIdx.x >> 5];
     TravStats st = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
     unsigned long long segs = 0;
-    const int lane = threadIdx.x & 31;
+    const BatchTile* tiles = P.tiles + P.mode_first[MODE];
+    const unsigned n = (unsigned)P.mode_tiles[MODE];
+    auto take = [&]() {  // index of the next tile, warp-uniform
+        unsigned t = 0u;
+        if ((threadIdx.x & 31) == 0) t = (unsigned)atomicAdd(P.work + MODE, 1ull);
+        return __shfl_sync(0xffffffffu, t, 0);
+    };
     TraceCtx C;
     C.nodes = P.nodes;
     C.qnodes = P.qnodes;
     C.tris = P.tris;
     C.max_visits = P.max_visits;
-    C.fetch = kFetchChunk;  // unused: each tile is one warp's whole pool
     C.ready = nullptr;
-    C.ready_chunk = 1;
-    C.wait_polls = kWaitPolls;
     C.order = nullptr;
     C.status = P.status;
-    while (true) {
-        unsigned long long t = 0ull;
-        if (lane == 0) t = atomicAdd(P.work + MODE, 1ull);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= (unsigned long long)P.mode_tiles[MODE]) break;
-        const BatchTile tile = P.tiles[P.mode_first[MODE] + t];
+    unsigned t = take();
+    while (t < n) {
+        const BatchTile tile = tiles[t];
         const BatchItemDev& it = P.items[tile.item];
         C.A = it.A;
         C.B = it.B;
@@ -102,7 +107,15 @@ __global__ void __maxnreg__(kWalkRegs) k_batch_walk(BatchParams P) {
         C.out = it.out;
         C.frame = P.frame + 2 * tile.item;
         C.coarse = it.n > 0 && walk_coarse(P.coarse[tile.item], it.n);
-        walk_loop<MODE, false, LEAFN>(C, sg, it.start, nullptr, tile.lo, tile.hi, st, segs);
+        auto next = [&](unsigned& pool, unsigned& pool_end) {
+            t = take();
+            if (t >= n || tiles[t].item != tile.item) return false;
+            pool = (unsigned)tiles[t].lo;
+            pool_end = (unsigned)tiles[t].hi;
+            return true;
+        };
+        walk_loop<MODE, false, LEAFN>(C, sg, it.start, (unsigned)tile.lo, (unsigned)tile.hi, true,
+                                      next, st, segs);
     }
 }
 

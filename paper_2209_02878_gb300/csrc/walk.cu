@@ -37,10 +37,12 @@ __global__ void __maxnreg__(kWalkRegs) k_walk(TraceParams P) {
     if (SMALL) {
         const int64_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
         const int64_t lo = min(P.nR, w * P.fetch);
-        walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, nullptr, lo, min(P.nR, lo + P.fetch), st,
+        walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, (unsigned)lo,
+                                      (unsigned)min(P.nR, lo + P.fetch), false, WalkNone{}, st,
                                       segs);
     } else {
-        walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, P.walk_work, 0, P.nR, st, segs);
+        walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, 0u, 0u, true, WalkCounter{C, P.walk_work}, st,
+                                      segs);
         walk_finish(P.walk_work);
     }
     if (STATS) flush_stats(st, P.stats, segs);

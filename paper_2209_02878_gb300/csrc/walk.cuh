@@ -66,6 +66,9 @@ constexpr int kTail = 4;
 // on the 1.31M-triangle sphere with 1M segments boolean 449 / 386 / 360 / 374,
 // count 780 / 700 / 673 / 713, nearest 654 / 661 / 610 / 637.
 constexpr int kWalkRegs = 80;
+// The batch's kernels hold an item's pointers as well: 80 / 96 / 112 / 128:
+// 1,215 / 1,143 / 1,180 / 1,151 us on 16 meshes with 3.5M segments.
+constexpr int kBatchRegs = 96;
 
 // Byte selectors that turn the low / high half of a node word into a float.
 constexpr unsigned kSelLo = 0x7104u, kSelHi = 0x7324u, kSelFar = kSelLo ^ kSelHi;
@@ -456,20 +459,20 @@ __device__ __forceinline__ unsigned walk_steps(const TraceCtx& C, const WalkSeg&
     return inner;
 }
 
-// Persistent per-warp loop over segments [lo, hi) (work distribution, order,
-// streamed input and compaction as trace_loop).  `start` is the first item
-// of every segment: the Karras root's slot, the whole mesh as one leaf, or
-// kNoRoot.  Must be called by all 32 lanes of the warp; sg is the warp's own.
-template <int MODE, bool STATS, bool LEAFN>
+// Persistent per-warp loop over the segments [pool, pool_end) and, while `more`,
+// those that next(pool, pool_end) fetches (it returns false when there are
+// none; warp-uniform); order, streamed input and compaction as in trace_loop.
+// Segment indices fit 31 bits (walk_fits).  `start` is the first item of every
+// segment: the Karras root's slot, the whole mesh as one leaf, or kNoRoot.
+// Must be called by all 32 lanes of the warp; sg is the warp's own.
+template <int MODE, bool STATS, bool LEAFN, typename Next>
 __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int start,
-                                          unsigned long long* counter, int64_t lo, int64_t hi,
-                                          TravStats& st, unsigned long long& segs) {
+                                          unsigned pool, unsigned pool_end, bool more,
+                                          const Next& next, TravStats& st,
+                                          unsigned long long& segs) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    // segment indices fit 31 bits (walk_fits)
-    unsigned pool = (unsigned)lo, pool_end = counter ? (unsigned)lo : (unsigned)hi;
-    bool more = counter != nullptr;  // the counter may hold more chunks
     int head = 0, avail = 0;         // staged segments not yet taken
     unsigned i = kNoBest;            // this lane's segment (kNoBest: none)
     int cur = kDone, sp = 0;
@@ -516,25 +519,8 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
             while (true) {
                 if (avail == 0) {  // set up the next segments, one per lane
                     if (pool >= pool_end) {
+                        more = more && next(pool, pool_end);
                         if (!more) break;
-                        unsigned long long b = 0ull;
-                        if (lane == 0) b = atomicAdd(counter, (unsigned long long)C.fetch);
-                        b = __shfl_sync(FULL, b, 0);
-                        if (b >= (unsigned long long)hi) {
-                            more = false;
-                            break;
-                        }
-                        pool = (unsigned)b;
-                        pool_end = (unsigned)min((long long)(b + C.fetch), (long long)hi);
-                        // streamed input: see trace_loop
-                        if (C.ready &&
-                            !wait_flag(C.ready + (int64_t)(pool_end - 1) / C.ready_chunk, C.status,
-                                       C.wait_polls)) {
-                            if (lane == 0) atomicMax(counter, (unsigned long long)hi);
-                            pool = pool_end;
-                            more = false;
-                            break;
-                        }
                     }
                     const int take = (int)min(pool_end - pool, 32u);
                     bool ok = false;
@@ -640,6 +626,33 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
         }
     }
 }
+
+// Source of segments of a launch over one mesh: chunks of C.fetch from a
+// counter.
+struct WalkCounter {
+    const TraceCtx& C;
+    unsigned long long* counter;
+    __device__ __forceinline__ bool operator()(unsigned& pool, unsigned& pool_end) const {
+        unsigned long long b = 0ull;
+        if ((threadIdx.x & 31) == 0) b = atomicAdd(counter, (unsigned long long)C.fetch);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (b >= (unsigned long long)C.nR) return false;
+        pool = (unsigned)b;
+        pool_end = (unsigned)min((long long)(b + C.fetch), (long long)C.nR);
+        // streamed input: see trace_loop
+        if (C.ready && !wait_flag(C.ready + (int64_t)(pool_end - 1) / C.ready_chunk, C.status,
+                                  C.wait_polls)) {
+            if ((threadIdx.x & 31) == 0) atomicMax(counter, (unsigned long long)C.nR);
+            pool = pool_end;
+            return false;
+        }
+        return true;
+    }
+};
+
+struct WalkNone {
+    __device__ __forceinline__ bool operator()(unsigned&, unsigned&) const { return false; }
+};
 
 // End of a block of a launch whose warps took work from counter[0]: the last
 // block clears it and the count of finished blocks (counter[1]) for the next
