@@ -79,7 +79,7 @@ __global__ void __maxnreg__(128) k_batch(BatchParams P) {
 template <int MODE, bool LEAFN>
 __global__ void __maxnreg__(kBatchRegs) k_batch_walk(BatchParams P) {
     extern __shared__ float4 stage4[];
-    WalkStage& sg = ((WalkStage*)stage4)[threadIdx.x >> 5];
+    WalkStage<false>& sg = ((WalkStage<false>*)stage4)[threadIdx.x >> 5];
     TravStats st = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
     unsigned long long segs = 0;
     const BatchTile* tiles = P.tiles + P.mode_first[MODE];
@@ -114,7 +114,7 @@ __global__ void __maxnreg__(kBatchRegs) k_batch_walk(BatchParams P) {
             pool_end = (unsigned)tiles[t].hi;
             return true;
         };
-        walk_loop<MODE, false, LEAFN>(C, sg, it.start, (unsigned)tile.lo, (unsigned)tile.hi, true,
+        walk_loop<MODE, false, LEAFN, false>(C, sg, it.start, (unsigned)tile.lo, (unsigned)tile.hi, true,
                                       next, st, segs);
     }
 }
@@ -158,7 +158,7 @@ static cudaError_t launch_batch_walk(const BatchParams& P, int block, cudaStream
         if (P.mode_tiles[mode] == 0) continue;
         BatchFn fn = batch_walk_kernel(mode, P.leaf_size > 1);
         const int bl = max_block((const void*)fn, block);
-        const int smem = (bl / 32) * (int)sizeof(WalkStage);
+        const int smem = (bl / 32) * (int)sizeof(WalkStage<false>);
         int grid = 0;
         cudaError_t e = occupancy_grid((const void*)fn, bl, smem, &grid);
         if (e != cudaSuccess) return e;

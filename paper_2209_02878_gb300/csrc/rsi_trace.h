@@ -141,6 +141,7 @@ struct BatchFork {
 
 using WalkFn = void (*)(TraceParams);
 WalkFn walk_kernel(int mode, bool stats, bool leafn, bool small);
+int walk_smem(int mode, int block);
 
 // Whether the phased loop (walk.cuh) can take nR segments against trees of n
 // triangles in all, and its first item for a mesh of n triangles at off.

@@ -159,7 +159,7 @@ cudaError_t launch_trace(const TraceParams& P, int mode, int stack, bool stats, 
                        : trace_kernel(mode, stack, stats, width, P.root < 0);
     const int block0 = block;
     block = max_block((const void*)fn, block);  // register-limited kernels cap the block
-    int smem = walk ? (block / 32) * (int)sizeof(WalkStage)
+    int smem = walk ? walk_smem(mode, block)
                     : P.smem_nodes > 0 ? P.smem_nodes * 64 : 0;
     int grid = 0;
     cudaError_t e = occupancy_grid((const void*)fn, block, smem, &grid);
@@ -175,7 +175,7 @@ cudaError_t launch_trace(const TraceParams& P, int mode, int stack, bool stats, 
     if (walk && !stats && !P.ready && P.nR <= 32 * warps) {
         fn = walk_kernel(mode, false, leafn, true);
         block = max_block((const void*)fn, block0);
-        smem = (block / 32) * (int)sizeof(WalkStage);
+        smem = walk_smem(mode, block);
         e = occupancy_grid((const void*)fn, block, smem, &grid);
         if (e != cudaSuccess) return e;
         warps = (int64_t)grid * (block / 32);

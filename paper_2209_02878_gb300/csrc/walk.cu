@@ -12,7 +12,7 @@ namespace rsi {
 // launches (10,000 segments over 1,922 triangles 53 -> 35 us), and the
 // triangle tests do not wait for lanes that a refill would have filled.
 template <int MODE, bool STATS, bool LEAFN, bool SMALL>
-__global__ void __maxnreg__(kWalkRegs) k_walk(TraceParams P) {
+__global__ void __maxnreg__(kWalkRegs<MODE>) k_walk(TraceParams P) {
     extern __shared__ float4 stage4[];
     TraceCtx C;
     C.A = P.A;
@@ -33,15 +33,16 @@ __global__ void __maxnreg__(kWalkRegs) k_walk(TraceParams P) {
     C.out = P.out;
     TravStats st = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
     unsigned long long segs = 0;
-    WalkStage& sg = ((WalkStage*)stage4)[threadIdx.x >> 5];
+    using Stage = WalkStage<kOwn<MODE>>;
+    Stage& sg = ((Stage*)stage4)[threadIdx.x >> 5];
     if (SMALL) {
         const int64_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
         const int64_t lo = min(P.nR, w * P.fetch);
-        walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, (unsigned)lo,
+        walk_loop<MODE, STATS, LEAFN, kOwn<MODE>>(C, sg, P.root, (unsigned)lo,
                                       (unsigned)min(P.nR, lo + P.fetch), false, WalkNone{}, st,
                                       segs);
     } else {
-        walk_loop<MODE, STATS, LEAFN>(C, sg, P.root, 0u, 0u, true, WalkCounter{C, P.walk_work}, st,
+        walk_loop<MODE, STATS, LEAFN, kOwn<MODE>>(C, sg, P.root, 0u, 0u, true, WalkCounter{C, P.walk_work}, st,
                                       segs);
         walk_finish(P.walk_work);
     }
@@ -59,6 +60,12 @@ WalkFn walk_kernel(int mode, bool stats, bool leafn, bool small) {
     if (stats) return leafn ? pick_walk<true, true, false>(mode) : pick_walk<true, false, false>(mode);
     if (small) return leafn ? pick_walk<false, true, true>(mode) : pick_walk<false, false, true>(mode);
     return leafn ? pick_walk<false, true, false>(mode) : pick_walk<false, false, false>(mode);
+}
+
+// Dynamic shared memory of a block.
+int walk_smem(int mode, int block) {
+    return block / 32 * (int)(mode == RSI_MODE_NEAREST ? sizeof(WalkStage<kOwn<RSI_MODE_NEAREST>>)
+                                                        : sizeof(WalkStage<kOwn<RSI_MODE_BOOL>>));
 }
 
 // 64-bit segment indices, and leaf references that do not fit an item (leaf

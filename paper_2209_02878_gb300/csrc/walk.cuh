@@ -61,13 +61,23 @@ constexpr int kStall = MODE == RSI_MODE_NEAREST ? 20 : 16;
 // still at work.
 constexpr int kTail = 4;
 
-// 80 registers (24 warps per SM): nothing of note spills.  64 / 72 / 80 / 88:
-// boolean 821 / 735 / 744 / 813 us, count 1,211 / 1,080 / 1,061 / 1,155 there;
-// on the 1.31M-triangle sphere with 1M segments boolean 449 / 386 / 360 / 374,
-// count 780 / 700 / 673 / 713, nearest 654 / 661 / 610 / 637.
-constexpr int kWalkRegs = 80;
-// The batch's kernels hold an item's pointers as well: 80 / 96 / 112 / 128:
-// 1,215 / 1,143 / 1,180 / 1,151 us on 16 meshes with 3.5M segments.
+// Whether a lane keeps its segment's end points and index, which node steps do
+// not need, in shared memory instead of seven registers, and the registers of
+// the kernels.  BOOL and COUNT then fit 72 without a spill (28 warps per SM):
+// 72 / 80 with, 64 / 72 / 80 / 88 without: boolean 697 / 758, 821 / 735 / 744 /
+// 813 us on the terrain above, 343 / 360, 449 / 386 / 360 / 374 on the
+// 1.31M-triangle sphere with 1M segments; count 994 / 1,058, 1,211 / 1,080 /
+// 1,061 / 1,155 and 619 / 664, 780 / 700 / 673 / 713.  NEAREST, which also needs
+// them for its outputs, does not gain: nearest of the raster 1,365 / 1,380
+// with, 1,437 / 1,400 / 1,345 without at 64 / 72 / 80, of the sphere 592 / 609
+// and 654 / 661 / 604.
+template <int MODE>
+constexpr bool kOwn = MODE != RSI_MODE_NEAREST;
+template <int MODE>
+constexpr int kWalkRegs = MODE == RSI_MODE_NEAREST ? 80 : 72;
+// The batch's kernels hold an item's pointers as well, and run side by side: 80 /
+// 96 / 112 / 128: 1,215 / 1,143 / 1,180 / 1,151 us on 16 meshes with 3.5M
+// segments; with the end points of boolean segments in shared memory 1,173.
 constexpr int kBatchRegs = 96;
 
 // Byte selectors that turn the low / high half of a node word into a float.
@@ -260,8 +270,11 @@ __device__ __forceinline__ bool walk_setup(const TraceCtx& C, int64_t i, WalkSeg
 
 // Segments set up by a warp and not yet taken by a lane (shared memory, one
 // per warp): four 16-byte words per segment.
+// And, with OWN, each lane's own segment {a, index}, {d, -}.
+template <bool OWN>
 struct WalkStage {
     float4 q[4][32];
+    float4 own[OWN ? 2 : 1][OWN ? 32 : 1];
 };
 
 // Best crossing of a NEAREST segment: leaf position (kBest64: decided in
@@ -465,8 +478,8 @@ __device__ __forceinline__ unsigned walk_steps(const TraceCtx& C, const WalkSeg&
 // Segment indices fit 31 bits (walk_fits).  `start` is the first item of every
 // segment: the Karras root's slot, the whole mesh as one leaf, or kNoRoot.
 // Must be called by all 32 lanes of the warp; sg is the warp's own.
-template <int MODE, bool STATS, bool LEAFN, typename Next>
-__device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int start,
+template <int MODE, bool STATS, bool LEAFN, bool OWN, typename Next>
+__device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage<OWN>& sg, int start,
                                           unsigned pool, unsigned pool_end, bool more,
                                           const Next& next, TravStats& st,
                                           unsigned long long& segs) {
@@ -474,12 +487,13 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     int head = 0, avail = 0;         // staged segments not yet taken
-    unsigned i = kNoBest;            // this lane's segment (kNoBest: none)
     int cur = kDone, sp = 0;
     int count = 0;                   // BOOL / COUNT: crossings
     unsigned best = kNoBest;         // NEAREST
     float tlo = 0.f, tlim = 1.f;     // NEAREST: bounds of the best crossing's t
     WalkSeg s;
+    int i = -1;                      // this lane's segment (-1: none)
+    if (OWN) sg.own[0][lane].w = i2f(-1);
     int stack[kWalkStack + 1];
     stack[0] = kDone;
     // node steps between two refills: each of the 32 segments takes at most
@@ -498,7 +512,8 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
             steps = 0;
             float dist = 0.f, P[3] = {0.f, 0.f, 0.f};
             Result res;
-            const bool fin = cur == kDone && i != kNoBest;
+            if (OWN) i = f2i(sg.own[0][lane].w);
+            const bool fin = cur == kDone && i >= 0;
             if (fin) {
                 if (MODE == RSI_MODE_BOOL) {
                     C.out.flag[i] = (uint8_t)(count > 0);
@@ -513,7 +528,10 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
             }
             if (MODE != RSI_MODE_BOOL && C.out.hit_idx)
                 compact<MODE>(C.out, fin && count > 0, i, res, dist, P);
-            if (fin) i = kNoBest;
+            if (fin) {
+                i = -1;
+                if (OWN) sg.own[0][lane].w = i2f(-1);
+            }
             if (!refillable) break;  // every lane is finished
             unsigned idle = dead;
             while (true) {
@@ -570,13 +588,18 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
                 if (cur == kDone && r < n) {
                     const float4 q0 = sg.q[0][head + r], q1 = sg.q[1][head + r];
                     const float4 q2 = sg.q[2][head + r], q3 = sg.q[3][head + r];
-                    s.ax_ = q0.x;
-                    s.ay_ = q0.y;
-                    s.az_ = q0.z;
-                    i = (unsigned)f2i(q0.w);
-                    s.dx = q1.x;
-                    s.dy = q1.y;
-                    s.dz = q1.z;
+                    if (OWN) {
+                        sg.own[0][lane] = q0;
+                        sg.own[1][lane] = q1;
+                    } else {
+                        s.ax_ = q0.x;
+                        s.ay_ = q0.y;
+                        s.az_ = q0.z;
+                        s.dx = q1.x;
+                        s.dy = q1.y;
+                        s.dz = q1.z;
+                        i = f2i(q0.w);
+                    }
                     s.fz = q1.w;
                     s.ix = q2.x;
                     s.iy = q2.y;
@@ -604,6 +627,16 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage& sg, int 
         if (nl > 0 && (nd + nl >= kStall<MODE> || inner == 0u || (!refillable && kTail * nl >= 32 - nd))) {
             // ---- triangle tests of the waiting leaves
             if (cur < 0 && cur != kDone) {
+                if (OWN) {  // the end points, for this phase only
+                    const float4 a = sg.own[0][lane], d = sg.own[1][lane];
+                    s.ax_ = a.x;
+                    s.ay_ = a.y;
+                    s.az_ = a.z;
+                    s.dx = d.x;
+                    s.dy = d.y;
+                    s.dz = d.z;
+                    i = f2i(a.w);
+                }
                 s.range();
                 const bool stop = walk_leaf<MODE, STATS, LEAFN>(C, s, i, cur, count, best, tlo,
                                                                 tlim, st);
