@@ -37,20 +37,20 @@ BYTES_PER_SEG_BOOL = 25     # 24 B of segment endpoints in + 1 B flag out
 BYTES_PER_SEG_NEAREST = 64  # 24 B in + tri, t, u, v, point, dist (40 B) out
 BYTES_PER_SEG_COUNT = 28
 # dram__bytes_read.sum + dram__bytes_write.sum and warp instructions of one
-# k_trace<BOOL> launch on this workload, from an ncu capture of the traversal
+# k_walk<BOOL> launch on this workload, from an ncu capture of the traversal
 # built from sources hashing to `sha`; reported as null once they differ
-TRAFFIC = {"sha": "9f8774bd7cbf58c6", "bytes": 257_930_240, "warp_inst": 953_680_560,
-           "l2_hit_pct": 81.7, "l1_hit_pct": 68.4}
+TRAFFIC = {"sha": "e1e309dfe8196ce2", "bytes": 258_327_296, "warp_inst": 535_331_909,
+           "l2_hit_pct": 73.0, "l1_hit_pct": 59.7}
 # peak warp-instruction issue rate: 152 SMs x 4 schedulers x 1 per cycle at
 # the maximum SM clock (2,070 MHz)
 ISSUE_PEAK = 152 * 4 * 2.070e9
-# FP32 operations the traversal performs per node visit (two child boxes, each
-# 6 subtract + 6 multiply + 4 max + 4 min + 1 multiply + 1 compare... counted
-# as 20) and per Moller-Trumbore test (~50); compared with the FP32 rate that
-# rsi_fp32_peak measures on the same GPU
-FP32_OPS_PER_VISIT = 40
+# FP32 operations the traversal performs per node visit (four boxes, each six
+# fused multiply-adds counted as two, two three-way maxima / minima counted as
+# two and a compare: 17) and per Moller-Trumbore test (~50); compared with the
+# FP32 rate that rsi_fp32_peak measures on the same GPU
+FP32_OPS_PER_VISIT = 68
 FP32_OPS_PER_TEST = 50
-TRAVERSAL_SOURCES = ("traverse_core.cuh", "rsi_internal.cuh", "traverse.cu")
+TRAVERSAL_SOURCES = ("walk.cuh", "walk.cu", "traverse_core.cuh", "rsi_internal.cuh", "traverse.cu")
 
 
 def traversal_sha():
@@ -222,11 +222,9 @@ def run_ours(args):
 
     with torch.cuda.stream(stream):
         bvh = rsi.BVH(V, T, stream=stream)
-        # build: bounds, Morton, 4 sort passes x (histogram, scatter; the scan
-        # is folded into the scatter at 30 tiles), Karras, climb; + traversal
-        # bounds, Morton, 4 x (histogram, scatter), Karras, the two box
+        # bounds, Morton, 4 x (histogram, scan, scatter), Karras, the two box
         # passes, the traversal
-        kernels_per_step = 2 + 2 * 4 + 1 + 2 + 1
+        kernels_per_step = 2 + 3 * 4 + 1 + 2 + 1
 
         def eager_step():
             bvh.build(V, T, stream=stream)
@@ -344,7 +342,7 @@ def run_ours(args):
         "config": {"workload": WORKLOAD, "n_triangles": mesh.n_tri, "segments_per_gpu": n_seg,
                    "parallelism": f"replicas x{world}, segments sharded per rank",
                    "l2": "inputs larger than L2 (240 MB of segments per step)",
-                   "launch": "persistent grid from occupancy, block 128, stack 64, binary nodes, "
+                   "launch": "persistent grid from occupancy, block 128, stack 64, four-way grid nodes, "
                              "input segment order, no shared-memory treelet",
                    "graph": not args.no_graph},
         "e2e": {"value": round(world * n_seg / (ms_e2e * 1e-3) / 1e6, 3), "unit": UNIT,
@@ -352,7 +350,7 @@ def run_ours(args):
                 "ms_per_step": round(ms_e2e, 4)},
         "gpu_launches": kernels_per_step * args.steps,
         "clocks": clk.summary(),
-        "roofline": {"bound": "hbm", "kernel": "k_trace<BOOL>", "achieved": round(achieved, 2),
+        "roofline": {"bound": "hbm", "kernel": "k_walk<BOOL>", "achieved": round(achieved, 2),
                      "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 5),
                      "peak_kind": peak_kind,
                      "traffic": TRAFFIC["bytes"] if traversal_sha() == TRAFFIC["sha"] else None,
@@ -360,12 +358,12 @@ def run_ours(args):
                      "l1_hit_pct": TRAFFIC["l1_hit_pct"] if traversal_sha() == TRAFFIC["sha"] else None,
                      "algorithmic_bytes_per_launch": algo_bytes,
                      "kernel_ms": round(ms_trav, 4)},
-        "issue_roofline": ({"bound": "issue", "kernel": "k_trace<BOOL>",
+        "issue_roofline": ({"bound": "issue", "kernel": "k_walk<BOOL>",
                             "achieved": round(TRAFFIC["warp_inst"] / (ms_trav * 1e-3) / 1e12, 4),
                             "peak": round(ISSUE_PEAK / 1e12, 4), "unit": "Twarp-inst/s",
                             "frac": round(TRAFFIC["warp_inst"] / (ms_trav * 1e-3) / ISSUE_PEAK, 4)}
                            if traversal_sha() == TRAFFIC["sha"] else None),
-        "fp32_roofline": {"bound": "fp32", "kernel": "k_trace<BOOL>",
+        "fp32_roofline": {"bound": "fp32", "kernel": "k_walk<BOOL>",
                           "achieved": round(fp32_ops / (ms_trav * 1e-3) / 1e12, 4),
                           "peak": round(fp32_tflops, 3), "unit": "TFLOP/s",
                           "frac": round(fp32_ops / (ms_trav * 1e-3) / 1e12 / fp32_tflops, 5),

@@ -110,8 +110,8 @@ typedef struct {
                            result; on height fields it avoids the splits
                            along the height that put both children across a
                            segment's path (131,072-triangle terrain,
-                           near-vertical segments: 29.2 -> 18.8 node visits,
-                           nearest 0.227 -> 0.127 ms).  Not in the paper. */
+                           near-vertical segments: 14.5 -> 9.5 node steps,
+                           nearest 0.110 -> 0.066 ms).  Not in the paper. */
 } rsi_build_opts;
 
 /* Options of one traversal launch.  Zero-initialised = defaults. */
@@ -139,13 +139,14 @@ typedef struct {
                             workspace of 16 B per segment, allocated by the
                             handle on first use (device allocator, on s) and
                             kept for later calls of the same or smaller nR. */
-    int32_t node_width;  /* traversal node arity: 2 (the binary tree, as in
-                            the paper) or 4 (each visit tests the four
-                            grandchildren of a binary node: half the chain of
-                            dependent node fetches, twice the box tests;
-                            its records are built by one extra kernel on the
-                            first 4-wide traversal after each build or
-                            refit); 0 -> 2.  smem_nodes > 0 implies 2. */
+    int32_t node_width;  /* 0 or 2: the default traversal, which takes two
+                            levels of the binary tree per step from records
+                            on a 15-bit grid (with stack_depth 64 and no
+                            treelet; else the paper's binary steps).  4: the
+                            four grandchildren with exact boxes, in records
+                            built by one extra kernel on the first such
+                            traversal after each build or refit (slower;
+                            smem_nodes > 0 overrides it). */
     int32_t packet;      /* 1: warp-cooperative traversal (f4, for coherent
                             segments): each warp takes 32 consecutive
                             segments in processing order and walks the tree
@@ -212,7 +213,8 @@ typedef struct {
 
 typedef struct {
     int64_t segments;
-    int64_t node_visits;   /* internal nodes fetched */
+    int64_t node_visits;   /* node records fetched (four boxes each on the
+                              default path, two on the general one) */
     int64_t tri_tests;     /* FP32 segment/triangle tests */
     int64_t fp64_tests;    /* tests decided by the FP64 recomputation */
     int64_t df_refines;    /* nearest hits whose outputs were recomputed in
@@ -265,8 +267,8 @@ rsi_status rsi_bvh_create(int64_t nV, int64_t nT, const rsi_build_opts* opt,
 /* Build the LBVH of (dV, dT) into h, asynchronously on s, without allocating
  * (capturable in a CUDA graph).  Steps (Sec. 2): centroid support interval,
  * 10-bit-per-axis quantisation and 30-bit Morton codes, on-device radix sort,
- * Karras binary radix tree, bottom-up boxes merged with per-node atomics
- * (Sec. 3.1 `atomic` field), optional leaf collapse and the top treelet.
+ * Karras binary radix tree, the boxes of the bottom-up pass (Sec. 3.1),
+ * optional leaf collapse and the top treelet.
  * dV float32[nV][3], dT int32[nT][3] with the sizes given at create time.
  * Index errors are latched for rsi_bvh_status.  Errors: RSI_ERR_ARG,
  * RSI_ERR_CUDA. */
@@ -341,7 +343,7 @@ rsi_status rsi_intersect(rsi_bvh h, const float* dA, const float* dB, int64_t nR
  * (DEVICE int32[nR], a permutation of [0, nR)) on s.  Uses the handle's
  * segment-order workspace (16 B per segment, allocated on first use from the
  * device allocator, on s).  Measured on 262,144 near-vertical segments over
- * a 131,072-triangle heightfield: nearest traversal 0.227 -> 0.185 ms against
+ * a 131,072-triangle heightfield: nearest traversal 0.110 -> 0.098 ms against
  * input order; random segments gain nothing.  Errors: RSI_ERR_ARG (NULL pointer,
  * nR < 0 or >= 2^31, bits out of range), RSI_ERR_NOT_BUILT, RSI_ERR_OOM,
  * RSI_ERR_CUDA. */
@@ -492,8 +494,9 @@ rsi_status rsi_batch_create(const rsi_batch_item* items, int32_t n,
  * Asynchronous, no allocation, capturable. */
 rsi_status rsi_batch_build(rsi_batch b, rsi_stream s);
 
-/* Traverse every item in ONE persistent launch (tiles pulled from an atomic
- * work counter, per-tile mode).  Asynchronous, no allocation, capturable. */
+/* Traverse every item: one persistent launch per mode (tiles pulled from an
+ * atomic work counter), side by side on the batch's own streams, which fork
+ * from s and join it again.  Asynchronous, no allocation, capturable. */
 rsi_status rsi_batch_intersect(rsi_batch b, rsi_stream s);
 
 /* Capture build + intersect of the batch into a CUDA graph once (on s) and

@@ -515,7 +515,7 @@ static rsi_status intersect_impl(rsi_bvh h, const float* dA, const float* dB, in
     else
         P.root = (int)(h->nT - 1);
     P.root4 = h->nT > 0 ? (int)(h->nT - 1) : rsi::kNoRoot;
-    P.leaf_size = h->leaf;
+    P.leaf_size = h->tb.leaf_size;  // of the built tree
     P.nT = (int)h->nT;
     P.nodes = h->tb.nodes;
     P.nodes4 = h->tb.nodes4;
@@ -550,7 +550,7 @@ static rsi_status intersect_impl(rsi_bvh h, const float* dA, const float* dB, in
         RSI_CK(cudaMemsetAsync(P.stats, 0, rsi::kStatCounters * 8, (cudaStream_t)s));
     // packets use the phased loop's items; meshes beyond those (walk_fits) get
     // the same results one segment per lane
-    if (c.packet && rsi::walk_fits(1, h->nT, h->leaf))
+    if (c.packet && rsi::walk_fits(1, h->nT, h->tb.leaf_size))
         RSI_CK(rsi::launch_trace_packet(P, mode, c.stats, (cudaStream_t)s));
     else
         RSI_CK(rsi::launch_trace(P, mode, c.stack, c.stats, c.block, c.width, (cudaStream_t)s));

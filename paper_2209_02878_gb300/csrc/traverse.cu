@@ -93,8 +93,8 @@ struct OccKey {
     int block, smem, dev;
 };
 static std::mutex g_occ_mu;
-static OccKey g_occ_key[64];
-static int g_occ_val[64];
+static OccKey g_occ_key[256];
+static int g_occ_val[256];
 static int g_occ_n = 0;
 
 int sm_count(int dev) {
@@ -131,7 +131,7 @@ cudaError_t occupancy_grid(const void* fn, int block, int smem, int* grid) {
     if (nb < 1) return cudaErrorInvalidConfiguration;
     const int g = nb * sm_count(dev);
     std::lock_guard<std::mutex> lk(g_occ_mu);
-    if (g_occ_n < 64) {
+    if (g_occ_n < 256) {
         g_occ_key[g_occ_n] = OccKey{fn, block, smem, dev};
         g_occ_val[g_occ_n] = g;
         ++g_occ_n;

@@ -30,15 +30,15 @@
 // so the decoding costs what that choice costs anyway.
 //
 // us: one loop for all / phases on exact binary nodes (64 B) / branch-free
-// steps on binary grid nodes (32 B) / on four-way grid nodes (64 B).  The
-// 29,768-triangle terrain with 10M random segments: boolean 1,177 / 1,010 /
-// 823 / 744, count 1,742 / 1,386 / 1,192 / 1,061, nearest 2,212 / 1,615 /
-// 1,426 / 1,336; nearest of its 10M-segment raster 2,291 / 1,498 / 1,387 /
-// 1,345; nearest of the 131,072-triangle terrain and 262,144 segments 238 /
-// 147 / 128 / 114; of the 1.31M-triangle sphere and 1M segments 1,100 / 796 /
-// 684 / 604, its count 1,172 / 965 / 773 / 665.  Boolean: warp instructions
-// 954M / 610M / 564M, L1 wavefronts 240M (65 % of the peak rate) / 253M (79 %) /
-// 148M (51 %), 14.4 / 22.9 / 23.8 active lanes, in the first three.
+// steps on binary grid nodes (32 B) / on four-way grid nodes (64 B) / with kOwn.
+// The 29,768-triangle terrain with 10M random segments: boolean 1,177 / 1,010 /
+// 823 / 744 / 697, count 1,742 / 1,386 / 1,192 / 1,061 / 995, nearest 2,212 /
+// 1,615 / 1,426 / 1,336 / -; nearest of its 10M-segment raster 2,291 / 1,498 /
+// 1,387 / 1,345 / -; nearest of the 131,072-triangle terrain and 262,144
+// segments 238 / 147 / 128 / 114 / -; of the 1.31M-triangle sphere and 1M
+// segments 1,100 / 796 / 684 / 604 / -, its count 1,172 / 965 / 773 / 665 / 617.
+// Boolean: warp instructions 954M / 610M / 564M / 528M, L1 wavefronts 65 % / 79 %
+// / 51 % / 54 % of the peak rate, 14.4 / 22.9 / 23.8 / 23.5 active lanes.
 #pragma once
 
 #include "traverse_core.cuh"
