@@ -27,8 +27,7 @@
 
 namespace rsi {
 
-// FUSED: hist[tile][d], so that the scatter's sums over the tiles read rows.
-template <typename K, int ITEMS, bool FUSED>
+template <typename K, int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const K* __restrict__ keys, int n,
                                                             int shift, uint32_t* __restrict__ hist,
                                                             int ntiles) {
@@ -46,8 +45,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const K* __restrict_
     for (int it = 0; it < ITEMS; ++it)
         if (dig[it] < kSortBins) atomicAdd(&h[dig[it]], 1u);
     __syncthreads();
-    hist[FUSED ? blockIdx.x * kSortBins + threadIdx.x : threadIdx.x * ntiles + blockIdx.x] =
-        h[threadIdx.x];
+    hist[threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
 // Block-wide exclusive scan of one value per thread (blockDim.x <= 1024).
@@ -97,7 +95,11 @@ static __global__ void __launch_bounds__(256) k_sort_scan(uint32_t* __restrict__
     if (threadIdx.x == 0) totals[blockIdx.x] = tot;
 }
 
-constexpr int kSortFuseTiles = 16;  // build of 29,768 triangles (30 tiles) 64 us fused, 60 not
+// The sums read the histograms a row per thread; tile-major histograms, whose
+// reads coalesce, measured slower (build of 29,768 triangles, 30 tiles: 64.5 us
+// against 69.8, and 66.5 with the scan kernel; at 64 tiles the sort of 65,536
+// keys takes 35 us with the scan kernel and 63 without).
+constexpr int kSortFuseTiles = 32;
 
 template <typename K, int ITEMS, bool FUSED>
 __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
@@ -119,10 +121,10 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
     // histograms) and the digit total; kSortThreads == bins, thread = digit
     uint32_t toff, dtot;
     if (FUSED) {
+        const uint32_t* row = hist + (size_t)threadIdx.x * ntiles;
         toff = dtot = 0u;
-#pragma unroll 8
         for (int q = 0; q < ntiles; ++q) {
-            const uint32_t x = hist[q * kSortBins + threadIdx.x];
+            const uint32_t x = row[q];
             toff += q < (int)blockIdx.x ? x : 0u;
             dtot += x;
         }
@@ -224,15 +226,13 @@ static cudaError_t radix_sort_tiles(K* keys[2], uint32_t* vals[2], int n, const 
     const int ntiles = (n + tile - 1) / tile;
     int cur = 0;
     for (int p = 0; p < np && n > 0; ++p) {
+        k_sort_hist<K, ITEMS><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p], hist,
+                                                              ntiles);
         if (ntiles <= kSortFuseTiles) {
-            k_sort_hist<K, ITEMS, true><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p],
-                                                                        hist, ntiles);
             k_sort_scatter<K, ITEMS, true><<<ntiles, kSortThreads, 0, s>>>(
                 keys[cur], vals[cur], keys[1 - cur], vals[1 - cur], n, shifts[p], hist, totals,
                 ntiles);
         } else {
-            k_sort_hist<K, ITEMS, false><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p],
-                                                                         hist, ntiles);
             k_sort_scan<<<kSortBins, 256, 0, s>>>(hist, ntiles, totals);
             k_sort_scatter<K, ITEMS, false><<<ntiles, kSortThreads, 0, s>>>(
                 keys[cur], vals[cur], keys[1 - cur], vals[1 - cur], n, shifts[p], hist, totals,
