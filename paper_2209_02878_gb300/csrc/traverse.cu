@@ -121,8 +121,14 @@ cudaError_t occupancy_grid(const void* fn, int block, int smem, int* grid) {
                 return cudaSuccess;
             }
     }
+    std::lock_guard<std::mutex> lk(g_occ_mu);
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        // the kernel's limit on this device only ever grows: a launch whose
+        // grid is in the cache does not come here to raise it again
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, fn);
+        if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes < smem)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
     int nb = 0;
@@ -130,7 +136,6 @@ cudaError_t occupancy_grid(const void* fn, int block, int smem, int* grid) {
     if (e != cudaSuccess) return e;
     if (nb < 1) return cudaErrorInvalidConfiguration;
     const int g = nb * sm_count(dev);
-    std::lock_guard<std::mutex> lk(g_occ_mu);
     if (g_occ_n < 256) {
         g_occ_key[g_occ_n] = OccKey{fn, block, smem, dev};
         g_occ_val[g_occ_n] = g;
