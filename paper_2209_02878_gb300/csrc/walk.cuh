@@ -42,6 +42,7 @@
 #pragma once
 
 #include "traverse_core.cuh"
+#include "walk_phase.h"
 
 namespace rsi {
 
@@ -57,9 +58,6 @@ constexpr int kWalkStack = 96;
 // 1,406 / 1,345 / 1,283 of its raster, 610 / 604 / 616 of the sphere.
 template <int MODE>
 constexpr int kStall = MODE == RSI_MODE_NEAREST ? 20 : 16;
-// The same once no segments are left to refill from: 1 / kTail of the lanes
-// still at work.
-constexpr int kTail = 4;
 
 // Whether a lane keeps its segment's end points and index, which node steps do
 // not need, in shared memory instead of seven registers, and the registers of
@@ -404,7 +402,7 @@ __device__ __forceinline__ void walk_nearest_out(const TraceCtx& C, const WalkSe
 }
 
 // The stack index is clamped, so that a corrupt tree cannot leave the array;
-// the step bound ends it.
+// the step bound (walk_more) ends its walk.
 __device__ __forceinline__ void walk_push(int* stack, int& sp, int x) {
     sp = min(sp + 1, kWalkStack);
     stack[sp] = x;
@@ -417,8 +415,8 @@ __device__ __forceinline__ void walk_push(int* stack, int& sp, int x) {
 // (as two binary steps would).
 template <int MODE, bool STATS, bool LEAFN, bool COARSE>
 __device__ __forceinline__ unsigned walk_steps(const TraceCtx& C, const WalkSeg& s, int& cur,
-                                               int& sp, int* stack, float tlim, unsigned& steps,
-                                               unsigned bound, int floor_, TravStats& st) {
+                                               int& sp, int* stack, float tlim, unsigned& left,
+                                               int floor_, TravStats& st) {
     constexpr bool LIMIT = MODE == RSI_MODE_NEAREST;
     unsigned inner;
     do {
@@ -468,7 +466,7 @@ __device__ __forceinline__ unsigned walk_steps(const TraceCtx& C, const WalkSeg&
             if (!any) cur = stack[sp--];
         }
         inner = __ballot_sync(0xffffffffu, cur >= 0);
-    } while (__popc(inner) > floor_ && ++steps < bound);
+    } while (walk_more(left, __popc(inner), floor_));
     return inner;
 }
 
@@ -496,20 +494,17 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage<OWN>& sg,
     if (OWN) sg.own[0][lane].w = i2f(-1);
     int stack[kWalkStack + 1];
     stack[0] = kDone;
-    // node steps between two refills: each of the 32 segments takes at most
-    // max_visits, so more can only be a corrupt tree
-    unsigned steps = 0;
-    const unsigned bound =
-        (unsigned)C.max_visits < 1u << 26 ? 32u * (unsigned)C.max_visits + 64u : 0xffffffffu;
+    unsigned left = walk_bound(C.max_visits);  // node steps until the next refill
     unsigned inner = 0u;  // lanes with a node step
     while (true) {
         const unsigned dead = __ballot_sync(FULL, cur == kDone);
         const unsigned leaf = ~(inner | dead);
         const bool refillable = avail > 0 || pool < pool_end || more;
         const int nd = __popc(dead), nl = __popc(leaf);
-        if (dead == FULL || (refillable && nd >= nl && nd + nl >= kStall<MODE>)) {
+        const WalkPhase phase = walk_phase(nd, nl, refillable, kStall<MODE>);
+        if (phase == kPhaseRefill) {
             // ---- refill: results of the finished segments, then new ones
-            steps = 0;
+            left = walk_bound(C.max_visits);
             float dist = 0.f, P[3] = {0.f, 0.f, 0.f};
             Result res;
             if (OWN) i = f2i(sg.own[0][lane].w);
@@ -624,7 +619,7 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage<OWN>& sg,
             inner = __ballot_sync(FULL, cur >= 0);
             continue;
         }
-        if (nl > 0 && (nd + nl >= kStall<MODE> || inner == 0u || (!refillable && kTail * nl >= 32 - nd))) {
+        if (phase == kPhaseLeaves) {
             // ---- triangle tests of the waiting leaves
             if (cur < 0 && cur != kDone) {
                 if (OWN) {  // the end points, for this phase only
@@ -647,12 +642,12 @@ __device__ __forceinline__ void walk_loop(const TraceCtx& C, WalkStage<OWN>& sg,
         }
         // ---- node steps until kStall lanes (a quarter of those left at the
         // end of the work) have none
-        const int floor_ = refillable ? 32 - kStall<MODE> : (32 - nd) - max(1, (31 + kTail - nd) / kTail);
-        inner = C.coarse ? walk_steps<MODE, STATS, LEAFN, true>(C, s, cur, sp, stack, tlim, steps,
-                                                                bound, floor_, st)
-                         : walk_steps<MODE, STATS, LEAFN, false>(C, s, cur, sp, stack, tlim, steps,
-                                                                 bound, floor_, st);
-        if (steps >= bound) {
+        const int floor_ = walk_floor(nd, refillable, kStall<MODE>);
+        inner = C.coarse ? walk_steps<MODE, STATS, LEAFN, true>(C, s, cur, sp, stack, tlim, left,
+                                                                floor_, st)
+                         : walk_steps<MODE, STATS, LEAFN, false>(C, s, cur, sp, stack, tlim, left,
+                                                                 floor_, st);
+        if (left == 0u) {
             if (lane == 0) atomicCAS(C.status, 0, RSI_ERR_INTERNAL);
             cur = kDone;
             inner = 0u;
