@@ -118,17 +118,20 @@ struct WalkSeg {
 // X(a) = base + (a - o) s and D = d s, with base = 1 on the grid and o = 0,
 // s = 1, base = 0 (exact) for the exact nodes; d = fl(b - a).
 // i = rcp.approx(D) (1 ulp) is (1 / D_exact)(1 + e), |e| <= 5u (d, D and the
-// reciprocal), and X(a) is off by at most 3u |X(a)| + 2u.  c = fl(X(a) i); a
-// face at X has the exact parameter (X - X_exact(a)) / D_exact, and X i - c is
-// that times (1 + e), up to 4u |c| + 2u |i|.  The constants are n = -(c + pad)
-// and f = pad - c with pad = 8u |c| + 4u |i| + 16u: the first two terms cover
-// those errors and the rounding of n / f (u |c|), and 16u the relative errors
-// e and the fma's own rounding for every parameter in [0, 1].  So for a box
+// reciprocal), and X(a) is off by at most 3u |X(a)| + 2u, or exact (s = 1).
+// c = fl(X(a) i); a face at X has the exact parameter (X - X_exact(a)) / D_exact,
+// and X i - c is that times (1 + e), up to 4u |c| + 2u |i| (exact nodes: u |c|).
+// The constants are n = -(c + pad) and f = pad - c with pad = 8u |c| + 4u |i| +
+// 16u: the first two terms cover those errors and the rounding of n / f (u |c|),
+// and 16u the relative errors e and the fma's own rounding for every parameter
+// in [0, 1].  The exact nodes go without 4u |i|: in their coordinates it would
+// move every face by 2.4e-7 whatever the mesh's size (segments 1e-5 long: 16
+// triangle tests each instead of 1.5; 2e-7 long: every triangle).  So for a box
 // that the exact segment meets at parameters [s0, s1] within [0, 1], the
 // computed entry is below s0 and the computed exit above s1, strictly, and
 // stays so after both are clamped to [0, 1]: `entry < exit` never rejects it.
 //  - |D| < 2^-62 (a zero component, and every tiny one): i = 2^62, pad = 2 +
-//    8u |c| + 4u i.  A segment inside the slab gets entry <= 0 and exit >= 1.
+//    8u |c| + 4u i (grid).  A segment inside the slab gets entry <= 0 and exit >= 1.
 //  - |D| > 2^100 (or infinite) or |c| > 2^100: i = 0, n = -2, f = 2: the
 //    axis never rejects.
 // Empty boxes: in the exact nodes both faces are +inf, which is always rejected
@@ -143,7 +146,7 @@ __device__ __forceinline__ void walk_axis(float a, float d, float o, float s, fl
     i = flat ? 0x1p62f : rcp_approx(D);
     const float c = __fmul_rn(X, i);
     const float pad = __fmaf_rn(fabsf(c), 0x1p-21f,
-                                __fmaf_rn(fabsf(i), 0x1p-22f, flat ? 2.f : 0x1p-20f));
+                                __fmaf_rn(fabsf(i), base * 0x1p-22f, flat ? 2.f : 0x1p-20f));
     n = -__fadd_rn(c, pad);
     f = __fsub_rn(pad, c);
     if (!(ad <= 0x1p100f && fabsf(c) <= 0x1p100f)) {
