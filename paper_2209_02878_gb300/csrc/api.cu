@@ -58,7 +58,7 @@ size_t carve(TreeBufs& tb, int64_t N, int M, int nblk, char* base) {
     tb.partial = (float*)take(4 * 12 * (size_t)(nblk > 0 ? nblk : 1));
     tb.bounds = (float*)take(4 * 6 * (size_t)M);
     tb.frame = (float4*)take(16 * 2 * (size_t)M);
-    tb.coarse = (int32_t*)take(4 * (size_t)M);
+    tb.coarse = (int2*)take(8 * (size_t)M);
     tb.rootbox = (float4*)take(16 * 2 * (size_t)M);
     tb.child = (int32_t*)take(4 * 2 * n1);
     tb.range = (int32_t*)take(4 * 2 * n1);

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kBuildThreads) k_bounds(MeshArgs ma, TreeBufs 
         if (!refit)
             for (int k = 0; k < 6; ++k) tb.bounds[6 * m + k] = v[k];
         write_frame(tb, m, v + 6, v + 9);
-        tb.coarse[m] = 0;
+        tb.coarse[m] = make_int2(0, 0);
         tb.done[m] = 0;
     }
 }
@@ -509,6 +509,44 @@ __device__ __forceinline__ void st_query(const float* st, int a, int b, float l[
     }
 }
 
+// Half the surface of a box in grid steps, its sides `out` steps longer (a
+// segment that passes a box meets one inside it with the ratio of their
+// surfaces as probability); 0 for an empty box.
+__device__ __forceinline__ float half_surface(const float l[3], const float h[3], const float s[3],
+                                              float out) {
+    if (l[0] > h[0]) return 0.f;
+    float e[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) e[k] = fmaxf((h[k] - l[k]) * s[k] * 32768.f, 0.f) + out;
+    return e[0] * (e[1] + e[2]) + e[1] * e[2];
+}
+
+// Whether the four-way nodes' grid blurs the leaf boxes of this warp's group
+// (rsi_internal.cuh), by their surfaces on the grid, about a step wider, and
+// exactly.  The whole warp calls it; groups with leaves of two meshes, or past
+// the last one, are left out.
+__device__ __forceinline__ void count_blurred(const TreeBufs& tb, const float* st, int m,
+                                              bool valid) {
+    const unsigned FULL = 0xffffffffu;
+    const int m0 = __shfl_sync(FULL, m, 0);
+    if (!__all_sync(FULL, valid && m == m0)) return;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const float4 s4 = tb.frame[2 * m + 1];
+    const float s[3] = {s4.x, s4.y, s4.z};
+    float l[3], h[3];
+    st_query(st, tid, tid, l, h);
+    float grid = half_surface(l, h, s, 1.f), exact = half_surface(l, h, s, 0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        grid += __shfl_xor_sync(FULL, grid, o);
+        exact += __shfl_xor_sync(FULL, exact, o);
+    }
+    if (lane != 0) return;
+    st_query(st, tid, tid + 31, l, h);
+    if (grid > kBlurDepth * half_surface(l, h, s, 1.f) && grid > kBlurRatio * exact)
+        atomicAdd(&tb.coarse[m].y, 32);
+}
+
 // a5, first pass.  One block per kBoxBlock consecutive sorted leaves, one
 // thread per leaf.  Each thread writes its triangle in leaf order and its
 // leaf box; the block builds a sparse table of its leaf boxes in shared
@@ -575,12 +613,10 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
         st[c * kStEntries + tid] = lo[c];
         st[(3 + c) * kStEntries + tid] = hi[c];
     }
-    {  // one atomic per warp and mesh
-        const unsigned cb = __ballot_sync(0xffffffffu, coarse);
-        if (cb) {
-            const unsigned peers = __match_any_sync(0xffffffffu, m) & cb;
-            if (coarse && lane == __ffs(peers) - 1) atomicAdd(tb.coarse + m, __popc(peers));
-        }
+    const unsigned fine = __ballot_sync(0xffffffffu, coarse);
+    if (fine) {  // one atomic per warp and mesh
+        const unsigned peers = __match_any_sync(0xffffffffu, m) & fine;
+        if (coarse && lane == __ffs(peers) - 1) atomicAdd(&tb.coarse[m].x, __popc(peers));
     }
     // slots whose range crosses a block boundary, for the second pass
     const bool inner = g < N && g - md.off < md.n - 1;  // an internal slot, not a root slot
@@ -615,6 +651,7 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
         }
     }
     __syncthreads();
+    if (fine) count_blurred(tb, st, m, md.n > 0);
     if (g >= N) return;
     float l0[3], h0[3];
     st_query(st, 0, tid, l0, h0);

@@ -64,7 +64,24 @@ constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
 constexpr int kSortTileMin = kSortThreads * 4;         // 1024 keys per tile (small sorts)
 constexpr int kSortBins = 256;
 constexpr int kBuildThreads = 256;
-constexpr float kCoarseSteps = 8.f;  // a leaf box below this many grid steps is coarse
+// Where the nodes' 15-bit grid is too coarse for a mesh: more than an eighth of
+// its leaf boxes are below kCoarseSteps steps, or more than kBlurredLeaves
+// leaves lie in groups of 32 (consecutive in leaf order) whose boxes it blurs
+// into one another: their surface grows over kBlurRatio times, which is how
+// many more of them a segment meets where they lie side by side, and over
+// kBlurDepth of them are met by a segment that passes the group (else they lie
+// far apart and cost little).
+// The second condition is for fine detail in a small part of a mesh: there the
+// cost of a segment grows with the triangles per grid cell (8,192 of 139,264
+// triangles in a patch 1e-5 wide: 4,308 tests and 9.9 ms for 20,000 segments,
+// 1.5 and 0.04 on the exact nodes).  kBlurRatio is a steep terrain with 1.3 grid
+// steps per quad.  20,000 boolean segments through 3,872 of 134,944 triangles at 0.45 /
+// 0.67 / 0.9 / 1.3 / 1.9 / 3.7 / 7.4 steps, us: on the grid 84, 58, 45, 41, 37, 30,
+// 27, on the exact nodes 41, 29, 27, 31, 31, 29, 29, in the general loop 43, 42,
+// 44, 55, 64, 52, 48; away from such detail the grid is the faster one (walk.cuh).
+constexpr float kCoarseSteps = 8.f;
+constexpr float kBlurDepth = 1.f, kBlurRatio = 2.5f;
+constexpr int kBlurredLeaves = 64;
 constexpr int kBoxBlock = 512;      // sorted leaves per block of the bottom-up box pass
 
 // FP32 filter constants (see mt32 below).
@@ -114,7 +131,7 @@ struct TreeBufs {
     float* partial;   // 12 * nblk: centroid and vertex intervals per block
     float* bounds;    // 6 * M
     float4* frame;    // 2 * M: grid of qnodes {origin, -}, {scale, -}
-    int32_t* coarse;  // M: leaves whose box spans fewer than kCoarseSteps grid steps
+    int2* coarse;     // M: leaves below kCoarseSteps grid steps, leaves in blurred groups
     int32_t* done;    // M: blocks of the mesh that k_bounds has finished (0 between launches)
     float4* rootbox;  // 2 * M: box of each mesh (lo, hi)
     int32_t* child;   // 2N

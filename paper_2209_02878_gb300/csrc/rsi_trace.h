@@ -30,8 +30,8 @@ struct TraceParams {
     const float4* nodes;
     const float4* nodes4;
     const float4* qnodes;  // phased loop: four-way records, their grid, and the
-    const float4* frame;   // number of leaves the grid is too coarse for
-    const int32_t* coarse;
+    const float4* frame;   // numbers of leaves that the grid is too coarse for
+    const int2* coarse;
     const float4* tris;
     const float4* treelet;
     const int32_t* treelet_n;
@@ -122,7 +122,7 @@ struct BatchParams {
     const float4* nodes4;
     const float4* qnodes;   // as in TraceParams, frame and coarse per item
     const float4* frame;
-    const int32_t* coarse;
+    const int2* coarse;
     const float4* tris;
     unsigned long long* work;
     int max_visits;

@@ -81,10 +81,11 @@ constexpr int kBatchRegs = 96;
 // Byte selectors that turn the low / high half of a node word into a float.
 constexpr unsigned kSelLo = 0x7104u, kSelHi = 0x7324u, kSelFar = kSelLo ^ kSelHi;
 
-// The nodes' grid (rsi_internal.cuh) has 32,760 steps across the mesh;
-// where more than an eighth of the leaf boxes are below kCoarseSteps steps
-// (fine detail in a far larger mesh) the loop reads the exact binary nodes.
-__device__ __forceinline__ bool walk_coarse(int coarse, int n) { return coarse > n / 8; }
+// The nodes' grid has 32,760 steps across the mesh; where that is too coarse for
+// its detail (rsi_internal.cuh) the loop reads the exact binary nodes.
+__device__ __forceinline__ bool walk_coarse(int2 coarse, int n) {
+    return coarse.x > n / 8 || coarse.y > kBlurredLeaves;
+}
 
 // A lane's segment: end points for the triangle test and, per axis, the
 // constants of the box test in the grid's coordinates
