@@ -7,8 +7,8 @@
 
 namespace rsi {
 
-// Enqueue the LBVH build (or, with refit, only the bottom-up box pass and the
-// treelet) of the meshes described by `ma` into the buffers of `tb` on s.
+// Enqueue the LBVH build (or, with refit, only the vertex bounds, the bottom-up
+// box pass and the treelet) of the meshes described by `ma` into the buffers of `tb` on s.
 cudaError_t build_tree(TreeBufs& tb, const MeshArgs& ma, cudaStream_t s, bool refit);
 
 // Raise the box pass's shared-memory limit on the current device (once per
