@@ -95,11 +95,14 @@ static __global__ void __launch_bounds__(256) k_sort_scan(uint32_t* __restrict__
     if (threadIdx.x == 0) totals[blockIdx.x] = tot;
 }
 
-// The sums read the histograms a row per thread; tile-major histograms, whose
-// reads coalesce, measured slower (build of 29,768 triangles, 30 tiles: 64.5 us
-// against 69.8, and 66.5 with the scan kernel; at 64 tiles the sort of 65,536
-// keys takes 35 us with the scan kernel and 63 without).
-constexpr int kSortFuseTiles = 32;
+// The sums read the histograms a row per thread.  us of a build (of a segment
+// order) as a graph, folded in / with the scan kernel, by tiles: 16: 55.7 / 56.9
+// (26.5 / 29.3), 20: 54.8 / 58.6 (26.6 / 32.3), 28: 58.7 / 60.1 (29.3 / 32.2), 32:
+// 69.7 / 59.5 (41.2 / 33.0), 36: 61.4 / 59.8 (31.5 / 32.8), 48: 73.1 / 62.5 (41.3 /
+// 32.5), 64: 89.2 / 63.3 (57.4 / 33.0): from 32 on the multiples of 16 tiles, whose
+// rows lie a multiple of 64 B apart, are the slowest.  (Tile-major histograms, whose reads coalesce:
+// build of 30 tiles 69.8 against 64.5.)
+constexpr int kSortFuseTiles = 31;
 
 template <typename K, int ITEMS, bool FUSED>
 __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
