@@ -59,9 +59,8 @@ namespace rsi {
 constexpr int kMaxLeaf = 8;
 constexpr int kTreeletMax = 2048;   // nodes in the breadth-first top treelet
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
-constexpr int kSortTileMin = kSortThreads * 4;         // 1024 keys per tile (small sorts)
+constexpr int kSortItems = 8;                   // keys per thread of a large sort
+constexpr int kSortTileMin = kSortThreads * 4;  // 1024 keys per tile (small sorts)
 constexpr int kSortBins = 256;
 constexpr int kBuildThreads = 256;
 // Where the nodes' 15-bit grid is too coarse for a mesh: more than an eighth of

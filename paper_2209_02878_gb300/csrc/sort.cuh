@@ -2,7 +2,7 @@
 // used for the triangle Morton keys (a3) and for the coherent segment order.
 //
 // One pass over digit `shift`:
-//   k_sort_hist    per tile of kSortTile keys: digit histogram -> hist[d][tile]
+//   k_sort_hist    per tile (radix_sort): digit histogram -> hist[d][tile]
 //   k_sort_scan    one block per digit: exclusive scan over the tiles of
 //                  hist[d][*] in place, digit total -> totals[d]
 //   k_sort_scatter per tile: digit bases (exclusive scan of totals), stable
@@ -10,7 +10,8 @@
 //                  ranks equal digits with __match_any_sync in key order),
 //                  scatter to base + tile offset + rank.
 // With at most kSortFuseTiles tiles the scan kernel is skipped: every
-// scatter block sums the (few) tile histograms of its digit itself.
+// scatter block sums the (few) tile histograms of its digit itself.  Tiles hold
+// 1,024 keys, those of large sorts 2,048 (radix_sort).
 //
 // What bounds the scatter is its stores: 35 us a pass at 1.31M 12-byte entries
 // when each lane stores to its own sector, 22 when the tile is ordered by digit
@@ -219,8 +220,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
 // keys[1] / vals[1] are ping-pong space; *out receives the index of the
 // buffer pair holding the result.  Tiles hold 1024 keys below 2^18 keys (more
 // blocks for small sorts: from 2^17 on, the build of 131,072 triangles takes 83
-// us instead of 78), 2048 above (4096: 362 against 359 us at 1.31M).  hist: kSortBins * ceil(n / 1024)
-// words, totals: kSortBins words.
+// us instead of 78), 2048 above (4096: 362 against 359 us at 1.31M).  hist:
+// kSortBins * ceil(n / 1024) words, totals: kSortBins words.
 template <typename K, int ITEMS>
 static cudaError_t radix_sort_tiles(K* keys[2], uint32_t* vals[2], int n, const int* shifts,
                                     int np, uint32_t* hist, uint32_t* totals, cudaStream_t s,
@@ -231,16 +232,13 @@ static cudaError_t radix_sort_tiles(K* keys[2], uint32_t* vals[2], int n, const 
     for (int p = 0; p < np && n > 0; ++p) {
         k_sort_hist<K, ITEMS><<<ntiles, kSortThreads, 0, s>>>(keys[cur], n, shifts[p], hist,
                                                               ntiles);
-        if (ntiles <= kSortFuseTiles) {
-            k_sort_scatter<K, ITEMS, true><<<ntiles, kSortThreads, 0, s>>>(
-                keys[cur], vals[cur], keys[1 - cur], vals[1 - cur], n, shifts[p], hist, totals,
-                ntiles);
-        } else {
+        auto scatter = k_sort_scatter<K, ITEMS, false>;
+        if (ITEMS <= 4 && ntiles <= kSortFuseTiles)  // large sorts always have more tiles
+            scatter = k_sort_scatter<K, ITEMS <= 4 ? ITEMS : 4, true>;
+        else
             k_sort_scan<<<kSortBins, 256, 0, s>>>(hist, ntiles, totals);
-            k_sort_scatter<K, ITEMS, false><<<ntiles, kSortThreads, 0, s>>>(
-                keys[cur], vals[cur], keys[1 - cur], vals[1 - cur], n, shifts[p], hist, totals,
-                ntiles);
-        }
+        scatter<<<ntiles, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[1 - cur],
+                                                vals[1 - cur], n, shifts[p], hist, totals, ntiles);
         cur = 1 - cur;
     }
     *out = cur;
