@@ -471,13 +471,7 @@ rsi_status rsi_bvh_export(rsi_bvh h, rsi_stream s, float* bounds, uint32_t* code
         rsi_status st = boxes(tb.lbox, N, lbox);
         if (st != RSI_OK) return st;
     }
-    if (nodes) {
-        RSI_CK(cudaMemcpy(nodes, tb.nodes, 64 * N, cudaMemcpyDeviceToHost));
-        int32_t* p = (int32_t*)nodes;
-        for (int64_t i = 0; i < N; ++i)  // leaf references are kept inverted on the device
-            for (int k = 12; k < 14; ++k)
-                if (p[16 * i + k + 2] > 0) p[16 * i + k] = ~p[16 * i + k];
-    }
+    if (nodes) RSI_CK(cudaMemcpy(nodes, tb.nodes, 64 * N, cudaMemcpyDeviceToHost));
     return RSI_OK;
 }
 

@@ -341,8 +341,8 @@ __device__ __forceinline__ void write_node(float4* nodes, int slot, float4 l0, f
     float f[16];
     store_child_box(l0, h0, f);
     store_child_box(l1, h1, f + 6);
-    f[12] = i2f(cnt0 > 0 ? ~ref0 : ref0);
-    f[13] = i2f(cnt1 > 0 ? ~ref1 : ref1);
+    f[12] = i2f(ref0);
+    f[13] = i2f(ref1);
     f[14] = i2f(cnt0);
     f[15] = i2f(cnt1);
     // the two children's coordinates interleaved in pairs (see rsi_internal.cuh)
@@ -418,10 +418,10 @@ __device__ __forceinline__ void binary_children(const float4* __restrict__ nodes
     a.hi[0] = f1.z; a.hi[1] = f2.x; a.hi[2] = f2.z;
     b.lo[0] = f0.y; b.lo[1] = f0.w; b.lo[2] = f1.y;
     b.hi[0] = f1.w; b.hi[1] = f2.y; b.hi[2] = f2.w;
+    a.ref = f2i(f3.x);
+    b.ref = f2i(f3.y);
     a.cnt = f2i(f3.z);
     b.cnt = f2i(f3.w);
-    a.ref = a.cnt > 0 ? ~f2i(f3.x) : f2i(f3.x);
-    b.ref = b.cnt > 0 ? ~f2i(f3.y) : f2i(f3.y);
 }
 
 // Expand binary slot `slot` (whose own record is already written) into its

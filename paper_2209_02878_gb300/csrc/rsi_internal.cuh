@@ -21,7 +21,7 @@
 //                      {c0.hi.y, c1.hi.y, c0.hi.z, c1.hi.z}
 //                      {ref0, ref1, cnt0, cnt1} as int bit patterns
 //                    cnt > 0: leaf of cnt triangles starting at sorted
-//                    position ~ref; cnt == 0: internal slot ref; cnt == -1:
+//                    position ref; cnt == 0: internal slot ref; cnt == -1:
 //                    treelet node ref (only inside the treelet copy).
 //                    Slot off+n-1 is the root slot (the paper keeps its root
 //                    pointer in internalNodes[N_t-1] the same way, Sec. 3.1):

@@ -214,8 +214,7 @@ __device__ __forceinline__ bool node_step(const TraceCtx& C, const Seg& s, int64
     float t0, t1;
     bool h0, h1;
     slab2(s, q0, q1, q2, tlim, h0, t0, h1, t1);
-    const int c0 = rc.z, c1 = rc.w;
-    const int r0 = c0 > 0 ? ~rc.x : rc.x, r1 = c1 > 0 ? ~rc.y : rc.y;
+    const int r0 = rc.x, r1 = rc.y, c0 = rc.z, c1 = rc.w;
     // one loop over both leaves for BOOL and COUNT; NEAREST keeps two (its
     // merged loop measured slower: more live state across the loop)
     if (MODE == RSI_MODE_NEAREST) {

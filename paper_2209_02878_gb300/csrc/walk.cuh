@@ -203,8 +203,7 @@ __device__ __forceinline__ bool walk_box(const WalkSeg& s, float ex, float ey, f
 // above 1), ~(8 position + count - 1).
 template <bool LEAFN>
 __device__ __forceinline__ int walk_item(int ref, int cnt) {
-    if (!LEAFN) return ref;
-    return cnt > 0 ? ~((~ref << 3) | (cnt - 1)) : ref;
+    return cnt > 0 ? ~(LEAFN ? ref << 3 | (cnt - 1) : ref) : ref;
 }
 
 // A node's children: whether the segment enters each, entry parameters and
