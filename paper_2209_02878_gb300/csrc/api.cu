@@ -471,7 +471,13 @@ rsi_status rsi_bvh_export(rsi_bvh h, rsi_stream s, float* bounds, uint32_t* code
         rsi_status st = boxes(tb.lbox, N, lbox);
         if (st != RSI_OK) return st;
     }
-    if (nodes) RSI_CK(cudaMemcpy(nodes, tb.nodes, 64 * N, cudaMemcpyDeviceToHost));
+    if (nodes) {
+        RSI_CK(cudaMemcpy(nodes, tb.nodes, 64 * N, cudaMemcpyDeviceToHost));
+        // the root slot's second child: no child (on the device: the null triangle)
+        int32_t* root = (int32_t*)nodes + 16 * (N - 1);
+        root[13] = -1;
+        root[15] = 0;
+    }
     return RSI_OK;
 }
 

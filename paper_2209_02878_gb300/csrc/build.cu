@@ -394,17 +394,19 @@ __device__ __forceinline__ void write_qnode(const TreeBufs& tb, int m, int slot,
     if (cnt1 > 0) write_half(tb, m, 2 * slot + 1, l1, h1, x1, e0, e1, none);
 }
 
+// none: position of the null triangle.
 __device__ __forceinline__ void write_root(float4* nodes, int slot, float4 lo, float4 hi, int ref,
-                                           int cnt) {
+                                           int cnt, int none) {
     const float4 e = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
-    write_node(nodes, slot, lo, hi, ref, cnt, e, e, -1, 0);
+    write_node(nodes, slot, lo, hi, ref, cnt, e, e, none, 1);
 }
 
 // 4-wide traversal node of slot `slot` (8 x float4 = 128 B, one record per
 // binary slot): the grandchildren of the binary node, i.e. each internal
 // child is replaced by its own two children, a leaf child is kept.  Layout:
 // {lo.x[4]}, {lo.y[4]}, {lo.z[4]}, {hi.x[4]}, {hi.y[4]}, {hi.z[4]},
-// {ref[4]}, {cnt[4]}; an empty slot has lo = hi = +inf, ref -1, cnt 0.
+// {ref[4]}, {cnt[4]}; an empty slot has lo = hi = +inf and the null triangle
+// (position `none`) as its leaf.
 struct Slot4 {
     float lo[3], hi[3];
     int ref, cnt;
@@ -427,7 +429,7 @@ __device__ __forceinline__ void binary_children(const float4* __restrict__ nodes
 // Expand binary slot `slot` (whose own record is already written) into its
 // 4-wide record.
 __device__ __forceinline__ void write_node4(const float4* __restrict__ nodes, float4* nodes4,
-                                            int slot) {
+                                            int slot, int none) {
     Slot4 c[2], o[4];
     binary_children(nodes, slot, c[0], c[1]);
     int k = 0;
@@ -441,8 +443,8 @@ __device__ __forceinline__ void write_node4(const float4* __restrict__ nodes, fl
     }
     for (; k < 4; ++k) {
         for (int a = 0; a < 3; ++a) o[k].lo[a] = o[k].hi[a] = INFINITY;
-        o[k].ref = -1;
-        o[k].cnt = 0;
+        o[k].ref = none;
+        o[k].cnt = 1;
     }
     float4* d = nodes4 + 8 * (int64_t)slot;
     for (int a = 0; a < 3; ++a) {
@@ -483,7 +485,7 @@ __device__ __forceinline__ void finish_node(const TreeBufs& tb, const MeshDesc& 
         const int root_slot = md.off + md.n - 1;
         tb.rootbox[2 * m] = f4(ul);
         tb.rootbox[2 * m + 1] = f4(uh);
-        write_root(tb.nodes, root_slot, f4(ul), f4(uh), md.off, md.n <= L ? md.n : 0);
+        write_root(tb.nodes, root_slot, f4(ul), f4(uh), md.off, md.n <= L ? md.n : 0, tb.N);
     }
 }
 
@@ -633,7 +635,7 @@ __global__ void __launch_bounds__(kBoxBlock) k_boxes_local(MeshArgs ma, TreeBufs
         }
         st2(tb.lbox + 2 * (int64_t)g, f4(lo), f4(hi));
         if (md.n == 1) {
-            write_root(tb.nodes, md.off, f4(lo), f4(hi), g, 1);
+            write_root(tb.nodes, md.off, f4(lo), f4(hi), g, 1, N);
             tb.rootbox[2 * m] = f4(lo);
             tb.rootbox[2 * m + 1] = f4(hi);
         }
@@ -835,7 +837,7 @@ __global__ void __launch_bounds__(128) k_boxes_span(MeshArgs ma, TreeBufs tb,
 // traversal, so it runs on first use.
 __global__ void k_nodes4(const float4* __restrict__ nodes, float4* __restrict__ nodes4, int N) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g < N) write_node4(nodes, nodes4, g);
+    if (g < N) write_node4(nodes, nodes4, g, N);
 }
 
 // ---------------------------------------------------------------- treelet
