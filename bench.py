@@ -39,8 +39,8 @@ BYTES_PER_SEG_COUNT = 28
 # dram__bytes_read.sum + dram__bytes_write.sum and warp instructions of one
 # k_walk<BOOL> launch on this workload, from an ncu capture of the traversal
 # built from sources hashing to `sha`; reported as null once they differ
-TRAFFIC = {"sha": "e1e309dfe8196ce2", "bytes": 258_327_296, "warp_inst": 535_331_909,
-           "l2_hit_pct": 73.0, "l1_hit_pct": 59.7}
+TRAFFIC = {"sha": "e09b10667290b26e", "bytes": 258_020_608, "warp_inst": 536_914_389,
+           "l2_hit_pct": 73.2, "l1_hit_pct": 59.9}
 # peak warp-instruction issue rate: 152 SMs x 4 schedulers x 1 per cycle at
 # the maximum SM clock (2,070 MHz)
 ISSUE_PEAK = 152 * 4 * 2.070e9
@@ -50,7 +50,8 @@ ISSUE_PEAK = 152 * 4 * 2.070e9
 # FP32 rate that rsi_fp32_peak measures on the same GPU
 FP32_OPS_PER_VISIT = 68
 FP32_OPS_PER_TEST = 50
-TRAVERSAL_SOURCES = ("walk.cuh", "walk.cu", "traverse_core.cuh", "rsi_internal.cuh", "traverse.cu")
+TRAVERSAL_SOURCES = ("walk.cuh", "walk_phase.h", "walk.cu", "traverse_core.cuh",
+                     "rsi_internal.cuh", "traverse.cu")
 
 
 def traversal_sha():

@@ -141,8 +141,10 @@ typedef struct {
                             kept for later calls of the same or smaller nR. */
     int32_t node_width;  /* 0 or 2: the default traversal, which takes two
                             levels of the binary tree per step from records
-                            on a 15-bit grid (with stack_depth 64 and no
-                            treelet; else the paper's binary steps).  4: the
+                            on a 15-bit grid, or exact binary steps where
+                            the grid is too coarse for a mesh's detail (with
+                            stack_depth 64 and no treelet; else the paper's
+                            binary steps).  4: the
                             four grandchildren with exact boxes, in records
                             built by one extra kernel on the first such
                             traversal after each build or refit (slower;
@@ -213,8 +215,11 @@ typedef struct {
 
 typedef struct {
     int64_t segments;
-    int64_t node_visits;   /* node records fetched (four boxes each on the
-                              default path, two on the general one) */
+    int64_t node_visits;   /* node records fetched: four boxes each on the
+                              default path and with node_width 4, two where
+                              the default path reads exact nodes (detail far
+                              below the mesh's size) and with the options
+                              that take binary steps */
     int64_t tri_tests;     /* FP32 segment/triangle tests */
     int64_t fp64_tests;    /* tests decided by the FP64 recomputation */
     int64_t df_refines;    /* nearest hits whose outputs were recomputed in
@@ -324,8 +329,8 @@ rsi_status rsi_bvh_export(rsi_bvh h, rsi_stream s, float* bounds, uint32_t* code
 
 /* Test nR segments (dA[i] -> dB[i]) against the tree in h (Sec. 3.2-3.3,
  * bvhIntersectionKernel): one persistent launch with warp-granular dynamic
- * work distribution, stack traversal testing both child boxes of each node
- * with a conservative slab test, triangles tested inline at the leaves.
+ * work distribution, stack traversal with conservative box tests, triangles
+ * tested at the leaves.
  * BOOL stops at the first crossing (Sec. 3.2, detected[rayIdx]); COUNT visits
  * every candidate; NEAREST prunes boxes beyond the best crossing so far.
  * out: see rsi_output.  lo: NULL = defaults.  nR == 0 is a no-op; an empty

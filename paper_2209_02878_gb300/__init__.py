@@ -488,7 +488,7 @@ def nearest_hit(V, T, A, B, bvh=None, order=None):
 
 class Batch:
     """Many independent (mesh, segments, mode) problems: one multi-mesh build
-    and one persistent traversal launch, optionally replayed as a CUDA graph
+    and one persistent traversal launch per mode, optionally replayed as a CUDA graph
     (rsi_batch_create / _build / _intersect / _run_graph).  Items are
     (V, T, A, B, mode) or (V, T, A, B, mode, height_axis); height_axis as for
     BVH, per item, or for every item without its own."""

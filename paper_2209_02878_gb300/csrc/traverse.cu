@@ -55,7 +55,6 @@ __global__ void __maxnreg__(TraceRegs<MODE>::value) k_trace(TraceParams P) {
     if (STATS) flush_stats(st, P.stats, segs);
 }
 
-// The default path (see walk.cuh).
 using KernelFn = void (*)(TraceParams);
 
 template <int MODE, bool STATS, int W, bool TL>
@@ -67,10 +66,10 @@ static KernelFn pick_stack(int stack) {
     }
 }
 
-// Without a treelet, BOOL and COUNT take the variant with the treelet tests
-// compiled out (1-2 % faster on the paper-scale heightfield); binary NEAREST
-// always takes the general one, which the register allocator handles better
-// (2.22 against 2.39 ms there).
+// Kernels of the general loop.  Without a treelet, BOOL and COUNT take the
+// variant with the treelet tests compiled out (1-2 % faster on the 29,768-
+// triangle heightfield); binary NEAREST always takes the one with them, which
+// the register allocator handles better (2.22 against 2.39 ms there).
 template <bool STATS, int W, bool TL>
 static KernelFn pick_mode(int mode, int stack) {
     if (mode == RSI_MODE_BOOL) return pick_stack<RSI_MODE_BOOL, STATS, W, TL>(stack);

@@ -1,16 +1,17 @@
-// Traversal loop of the default path: one segment per lane, binary nodes,
-// the whole tree in global memory (no treelet copy), a 64-entry stack.
-// traverse_core.cuh holds the general loop that serves the other options.
+// Traversal loop of the default path: one segment per lane, over four-way
+// records of the tree (exact binary nodes where those are too coarse), all in
+// global memory.  traverse_core.cuh holds the general loop that serves the
+// other options: smaller stacks, 4-wide exact nodes, treelets.
 //
 // What bounds it is instruction issue, the divergence between lanes and L1
 // wavefronts (one per 32-byte sector that a lane reads), not DRAM bytes (the
 // tree sits in L1 / L2).
 //
 // So the loop is split into three phases that each run with many lanes at
-// once:
-//  - node steps: every lane whose current item is a node tests the node's two
-//    child boxes and moves on (leaf children are items like nodes: entered
-//    or pushed, not tested here);
+// once (which one is next: walk_phase.h):
+//  - node steps: every lane whose current item is a node tests the node's
+//    four child boxes and moves on (leaf children are items like nodes:
+//    entered or pushed, not tested here);
 //  - triangle tests: lanes whose current item is a leaf wait until several of
 //    them do (inline, the test ran for 1.2 of 32 lanes on average);
 //  - refill: finished lanes write their results together and take new
@@ -18,27 +19,22 @@
 // A phase runs when kStall lanes cannot take a node step, the one with more
 // lanes waiting first.  NEAREST keeps only the best crossing's position and
 // interval across the loop (its outputs are recomputed once, when written),
-// which takes its spills away.
+// which leaves it 68 B of spills at 80 registers (166 in the general loop).
 //
-// And a node step takes two levels of the tree at once, from a 64-byte record
-// of the four grandchildren's boxes on a 15-bit grid over the mesh's box: as
-// many bytes and boxes per segment as binary steps on 32-byte grid nodes, but
-// half the steps, each of which costs a ballot, the stack and the loop beside
-// its boxes, and half the chain of dependent reads.  (Exact boxes take twice
-// the bytes.)  The 16-bit half that holds a face becomes a float in [1, 2) by
-// one byte permutation, whose selector also chooses the near or the far face,
-// so the decoding costs what that choice costs anyway.
+// And a node step takes two levels of the binary tree at once, from a 64-byte
+// record of the four grandchildren's boxes on a 15-bit grid over the mesh's
+// box: as many bytes and boxes per segment as binary steps on 32-byte grid
+// nodes, but half the steps, each of which costs a ballot, the stack and the
+// loop beside its boxes, and half the chain of dependent reads.  (Exact boxes
+// take twice the bytes.)  The 16-bit half that holds a face becomes a float in
+// [1, 2) by one byte permutation, whose selector also chooses the near or the
+// far face, so the decoding costs what that choice costs anyway.
 //
-// us: one loop for all / phases on exact binary nodes (64 B) / branch-free
-// steps on binary grid nodes (32 B) / on four-way grid nodes (64 B) / with kOwn.
-// The 29,768-triangle terrain with 10M random segments: boolean 1,177 / 1,010 /
-// 823 / 744 / 697, count 1,742 / 1,386 / 1,192 / 1,061 / 995, nearest 2,212 /
-// 1,615 / 1,426 / 1,336 / -; nearest of its 10M-segment raster 2,291 / 1,498 /
-// 1,387 / 1,345 / -; nearest of the 131,072-triangle terrain and 262,144
-// segments 238 / 147 / 128 / 114 / -; of the 1.31M-triangle sphere and 1M
-// segments 1,100 / 796 / 684 / 604 / -, its count 1,172 / 965 / 773 / 665 / 617.
-// Boolean: warp instructions 954M / 610M / 564M / 528M, L1 wavefronts 65 % / 79 %
-// / 51 % / 54 % of the peak rate, 14.4 / 22.9 / 23.8 / 23.5 active lanes.
+// us, general loop -> this one: 10M random segments over a 29,768-triangle
+// terrain boolean 1,179 -> 708, count 1,780 -> 1,021, nearest 2,202 -> 1,330,
+// nearest of its raster 2,317 -> 1,386; 1M segments over a 1.31M-triangle sphere
+// boolean 536 -> 283, count 1,462 -> 749, nearest 1,075 -> 601.  Boolean on the
+// terrain: warp instructions 954M -> 535M, active lanes 14.4 -> 23.3.
 #pragma once
 
 #include "traverse_core.cuh"
@@ -61,14 +57,10 @@ constexpr int kStall = MODE == RSI_MODE_NEAREST ? 20 : 16;
 
 // Whether a lane keeps its segment's end points and index, which node steps do
 // not need, in shared memory instead of seven registers, and the registers of
-// the kernels.  BOOL and COUNT then fit 72 without a spill (28 warps per SM):
-// 72 / 80 with, 64 / 72 / 80 / 88 without: boolean 697 / 758, 821 / 735 / 744 /
-// 813 us on the terrain above, 343 / 360, 449 / 386 / 360 / 374 on the
-// 1.31M-triangle sphere with 1M segments; count 994 / 1,058, 1,211 / 1,080 /
-// 1,061 / 1,155 and 619 / 664, 780 / 700 / 673 / 713.  NEAREST, which also needs
-// them for its outputs, does not gain: nearest of the raster 1,365 / 1,380
-// with, 1,437 / 1,400 / 1,345 without at 64 / 72 / 80, of the sphere 592 / 609
-// and 654 / 661 / 604.
+// the kernels.  BOOL then fits 72 without a spill and COUNT with 4 B (28 warps
+// per SM): boolean on the terrain above 697 us, 744 at 80 registers without;
+// count 994 and 1,061.  NEAREST, which also needs them for its outputs, does
+// not gain: nearest of the raster 1,365 us with at its best, 1,345 without.
 template <int MODE>
 constexpr bool kOwn = MODE != RSI_MODE_NEAREST;
 template <int MODE>
