@@ -111,7 +111,7 @@ typedef struct {
                            along the height that put both children across a
                            segment's path (131,072-triangle terrain,
                            near-vertical segments: 14.5 -> 9.5 node steps,
-                           nearest 0.110 -> 0.066 ms).  Not in the paper. */
+                           nearest 0.107 -> 0.066 ms).  Not in the paper. */
 } rsi_build_opts;
 
 /* Options of one traversal launch.  Zero-initialised = defaults. */
@@ -348,7 +348,7 @@ rsi_status rsi_intersect(rsi_bvh h, const float* dA, const float* dB, int64_t nR
  * (DEVICE int32[nR], a permutation of [0, nR)) on s.  Uses the handle's
  * segment-order workspace (16 B per segment, allocated on first use from the
  * device allocator, on s).  Measured on 262,144 near-vertical segments over
- * a 131,072-triangle heightfield: nearest traversal 0.110 -> 0.098 ms against
+ * a 131,072-triangle heightfield: nearest traversal 0.107 -> 0.097 ms against
  * input order; random segments gain nothing.  Errors: RSI_ERR_ARG (NULL pointer,
  * nR < 0 or >= 2^31, bits out of range), RSI_ERR_NOT_BUILT, RSI_ERR_OOM,
  * RSI_ERR_CUDA. */
